@@ -36,7 +36,14 @@ enum { kProfRaygen = 0, kProfTrace = 1, kProfShade = 2, kProfShadow = 3, kProfAc
     if (rc_ != ET_OK) return rc_;    \
   } while (0)
 
-enum { C_NRAY0 = 0, C_NRAY1 = 1, C_NSH = 2, C_FETCH = 3, C_FETCH_SH = 4, C_N = 8 };
+// Queue counters: one set per path segment, each counter in its own 128-byte
+// line (the appends and fetches of a kernel then meet in different L2 slices),
+// all cleared by one memset per batch.
+enum { C_NRAY = 0, C_NSH = 1, C_FETCH = 2, C_FETCH_SH = 3 };
+constexpr int kCtrLine = 32;
+constexpr int kMaxSegments = 16;     // max_depth
+constexpr int kCtrWords = 4 * kCtrLine * (kMaxSegments + 2);   // segments 1 .. 16 and the queue after the last
+__host__ __device__ __forceinline__ int ctr_of(int b, int kind) { return (4 * b + kind) * kCtrLine; }
 
 struct Batch {
   int f0, nf;          // frames of the call in this batch (relative to the call)
@@ -152,7 +159,7 @@ __device__ __forceinline__ uint32_t warp_append(uint32_t* counter, bool want) {
 
 __global__ void __launch_bounds__(256) wf_raygen(Args A) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q == 0) A.ctr[C_NRAY0] = (uint32_t)A.bt.paths;
+  if (q == 0) A.ctr[ctr_of(1, C_NRAY)] = (uint32_t)A.bt.paths;
   if (q >= A.bt.paths) return;
   int f, s;
   int64_t pix;
@@ -172,63 +179,39 @@ __global__ void __launch_bounds__(256) wf_raygen(Args A) {
 
 // Persistent traversal with dynamic ray fetch.  kShadow: any-hit shadow rays
 // (queue sho/shd/shc), else closest-hit extension rays (queue qo/qd -> hit).
-// resident blocks of 128 threads per SM the register allocation aims for
-#ifndef ET_TRACE_MIN_BLOCKS
-#define ET_TRACE_MIN_BLOCKS 12
-#endif
+// Bound by issue slots and L1 data reads of scattered nodes (ncu, 640x360 city,
+// second segment: 0.72 warp instructions per scheduler and cycle with 13 of 32
+// lanes active, L1 data stage 82 % busy).  Writing a result and taking a new
+// ray costs a warp about as much as several node visits and a queue round trip
+// however few lanes do it, so a warp waits until kRefill lanes are idle (4
+// frames of 720p: 11.60 ms at 8 lanes, 11.24 at 16, 11.10 at 20, 11.23 at 24),
+// and takes rays in stretches of its own: its first 32 without an atomic (the
+// Cornell box at 64 x 64 fits in these: 0.244 -> 0.210 ms per 8 frames), then
+// 32 at a time (64 and 128 at a time leave longer tails: +3 % and +11 % on the
+// 256 x 256 procedural scene).
+// Resident blocks of 128 threads per SM the register allocation aims for: 12
+// (10: equal; 14 spills, +5 %).
+constexpr int kTraceMinBlocks = 12;
+constexpr int kRefill = 20;
+constexpr uint32_t kChunk = 32;
 template <bool kShadow>
-__global__ void __launch_bounds__(128, ET_TRACE_MIN_BLOCKS) wf_trace(Args A, int cur, int b) {
-  const uint32_t n = A.ctr[kShadow ? C_NSH : (C_NRAY0 + cur)];
-  uint32_t* fetch = A.ctr + (kShadow ? C_FETCH_SH : C_FETCH);
+__global__ void __launch_bounds__(128, kTraceMinBlocks) wf_trace(Args A, int cur, int b) {
+  const uint32_t n = A.ctr[ctr_of(b, kShadow ? C_NSH : C_NRAY)];
+  uint32_t* fetch = A.ctr + ctr_of(b, kShadow ? C_FETCH_SH : C_FETCH);
   const unsigned lane = threadIdx.x & 31u;
   pt::Traversal<kShadow> tr;
   pt::Ray ray;
-  int idx = -1;                       // -1: wants a ray, -2: queue exhausted
+  int idx = -1;                       // queue index of the lane's ray, -1: none
+  // the warp's own stretch of the queue [pool, pool_end): the first 32 rays
+  // without an atomic, the k-th warp of every block before the (k + 1)-th so
+  // that a short queue spreads over all SMs; then kChunk at a time
+  const uint32_t n_static = gridDim.x * (blockDim.x >> 5) * 32u;
+  uint32_t pool = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32u, pool_end = pool + 32u;
   while (true) {
-    const unsigned want = __ballot_sync(FULL, idx == -1);
-    if (want) {
-      const int leader = __ffs(want) - 1;
-      uint32_t base = 0;
-      if ((int)lane == leader) base = atomicAdd(fetch, (uint32_t)__popc(want));
-      base = __shfl_sync(FULL, base, leader);
-      if (idx == -1) {
-        const uint32_t my = base + (uint32_t)__popc(want & ((1u << lane) - 1u));
-        if (my < n) {
-          idx = (int)my;
-          float4 o, d;
-          if (kShadow) { o = A.sho[my]; d = A.shd[my]; }
-          else {
-            if (A.perm) idx = (int)A.perm[my];
-            o = A.qo[cur][idx]; d = A.qd[cur][idx];
-          }
-          pt::ray_setup(ray, mk(o.x, o.y, o.z), mk(d.x, d.y, d.z));
-          tr.start(A.S, kShadow ? d.w : FLT_MAX);
-        } else {
-          idx = -2;
-        }
-      }
-    }
-    if (__all_sync(FULL, idx == -2)) break;
-    // node phase: lanes at inner nodes descend together; it ends when no lane
-    // has node work left or when enough lanes are waiting at a leaf
-    while (true) {
-      const bool node = idx >= 0 && tr.at_node();
-      const unsigned nodes = __ballot_sync(FULL, node);
-      if (!nodes) break;
-      const unsigned leaves = __ballot_sync(FULL, idx >= 0 && tr.at_leaf());
-      if (__popc(leaves) >= kLeafBatch) break;
-      // up to kNodeSteps steps per vote: a lane keeps descending while it is at
-      // an inner node (its own sequence of visits is unchanged)
-      if (node) {
-#pragma unroll
-        for (int r = 0; r < kNodeSteps; ++r)
-          if (tr.at_node()) tr.visit_node(A.S, ray);
-      }
-    }
-    // leaf phase: lanes at a leaf test its triangles together
-    if (idx >= 0 && tr.at_leaf()) tr.visit_leaf(A.S, ray);
-    {
-      if (idx >= 0 && tr.ref == pt::Traversal<kShadow>::kDone) {
+    const bool fin = idx >= 0 && tr.ref == pt::Traversal<kShadow>::kDone;
+    const unsigned idle = __ballot_sync(FULL, idx < 0 || fin);
+    if (__popc(idle) >= kRefill) {
+      if (fin) {
         if (kShadow) {
           const bool vis = tr.h.slot < 0;
           const float4 c = A.shc[idx];
@@ -249,12 +232,65 @@ __global__ void __launch_bounds__(128, ET_TRACE_MIN_BLOCKS) wf_trace(Args A, int
         }
         idx = -1;
       }
+      if (pool < n) {
+        const uint32_t cnt = (uint32_t)__popc(idle), have = pool_end - pool;
+        const uint32_t rank = (uint32_t)__popc(idle & ((1u << lane) - 1u));
+        uint32_t my = pool + rank;
+        if (have >= cnt) {
+          pool += cnt;
+        } else {
+          uint32_t nb = n_static;
+          if (n_static < n) {
+            if (lane == 0) nb += atomicAdd(fetch, kChunk);
+            nb = __shfl_sync(FULL, nb, 0);
+          }
+          if (rank >= have) my = nb + (rank - have);
+          pool = nb + (cnt - have);
+          pool_end = nb + kChunk;
+        }
+        if (((idle >> lane) & 1u) && my < n) {
+          idx = (int)my;
+          float4 o, d;
+          if (kShadow) { o = A.sho[my]; d = A.shd[my]; }
+          else {
+            if (A.perm) idx = (int)A.perm[my];
+            o = A.qo[cur][idx]; d = A.qd[cur][idx];
+          }
+          pt::ray_setup(ray, mk(o.x, o.y, o.z), mk(d.x, d.y, d.z));
+          tr.start(A.S, kShadow ? d.w : FLT_MAX);
+        }
+      }
+      if (__all_sync(FULL, idx < 0)) {
+        if (pool >= n) break;
+        continue;
+      }
     }
+    // node phase: lanes at inner nodes descend together; it ends when no lane
+    // has node work left or when enough lanes are waiting at a leaf
+    while (true) {
+      const bool node = idx >= 0 && tr.at_node();
+      const unsigned nodes = __ballot_sync(FULL, node);
+      if (!nodes) break;
+      const unsigned leaves = __ballot_sync(FULL, idx >= 0 && tr.at_leaf());
+      if (__popc(leaves) >= kLeafBatch) break;
+      // up to kNodeSteps steps per vote: a lane keeps descending while it is at
+      // an inner node (its own sequence of visits is unchanged)
+      if (node) {
+#pragma unroll
+        for (int r = 0; r < kNodeSteps; ++r)
+          if (tr.at_node()) tr.visit_node(A.S, ray);
+      }
+    }
+    // leaf phase: lanes at a leaf test its triangles together
+    if (idx >= 0 && tr.at_leaf()) tr.visit_leaf(A.S, ray);
   }
 }
 
-__global__ void __launch_bounds__(256) wf_shade(Args A, int cur, int b) {
-  const uint32_t n = A.ctr[C_NRAY0 + cur];
+// Bound by the latency of its gathers (ray, hit, triangle, path state): 64
+// registers for 4 blocks per SM instead of 76 for 3 (4 frames of 720p: 11.10 ->
+// 11.03 ms; 5 blocks spill, 11.24), launched 16 blocks per SM deep.
+__global__ void __launch_bounds__(256, 4) wf_shade(Args A, int cur, int b) {
+  const uint32_t n = A.ctr[ctr_of(b, C_NRAY)];
   const int nxt = cur ^ 1;
   // whole warps iterate together so that the appends can use warp ballots
   const uint32_t warp_id = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -297,13 +333,13 @@ __global__ void __launch_bounds__(256) wf_shade(Args A, int cur, int b) {
         if (want_ray) A.beta_pdf[q] = make_float4(beta.x, beta.y, beta.z, pdf);
       }
     }
-    const uint32_t js = warp_append(A.ctr + C_NSH, want_sh);
+    const uint32_t js = warp_append(A.ctr + ctr_of(b, C_NSH), want_sh);
     if (want_sh) {
       A.sho[js] = make_float4(v.on.x, v.on.y, v.on.z, __uint_as_float(q));
       A.shd[js] = make_float4(sh_dir.x, sh_dir.y, sh_dir.z, sh_tmax);
       A.shc[js] = make_float4(contrib.x, contrib.y, contrib.z, __uint_as_float((uint32_t)light));
     }
-    const uint32_t jr = warp_append(A.ctr + C_NRAY0 + nxt, want_ray);
+    const uint32_t jr = warp_append(A.ctr + ctr_of(b + 1, C_NRAY), want_ray);
     if (want_ray) {
       A.qo[nxt][jr] = make_float4(v.on.x, v.on.y, v.on.z, __uint_as_float(q));
       A.qd[nxt][jr] = make_float4(d_next.x, d_next.y, d_next.z, 0.0f);
@@ -344,7 +380,7 @@ int ensure_workspace(et_scene* s, int64_t paths, int64_t acc_pix) {
   s->wf_mem = nullptr;
   s->wf_cap = s->wf_acc_cap = 0;
   const int64_t cap = std::max<int64_t>(paths, 1), acap = std::max<int64_t>(acc_pix, 1);
-  const size_t bytes = (size_t)cap * (16 * 2 + 16 * 4 + 8 + 16 * 3) + (size_t)acap * 16 + 256;
+  const size_t bytes = (size_t)cap * (16 * 2 + 16 * 4 + 8 + 16 * 3) + (size_t)acap * 16 + sizeof(uint32_t) * kCtrWords + 256;
   ET_CHECK_CUDA(cudaMalloc(&s->wf_mem, bytes));
   s->wf_cap = cap;
   s->wf_acc_cap = acap;
@@ -423,7 +459,7 @@ int et_render_wavefront(et_scene* s, int n_frames, int first_frame, int W, int H
   A.shc = reinterpret_cast<float4*>(p); p += 16 * cap;
   float4* acc = reinterpret_cast<float4*>(p); p += 16 * s->wf_acc_cap;
   A.hit = reinterpret_cast<int2*>(p); p += 8 * cap;
-  A.ctr = reinterpret_cast<uint32_t*>(p);
+  A.ctr = reinterpret_cast<uint32_t*>((reinterpret_cast<uintptr_t>(p) + 127) & ~(uintptr_t)127);
   int dev = 0, nsm = 0, occ_c = 0, occ_s = 0;
   ET_CHECK_CUDA(cudaGetDevice(&dev));
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -442,7 +478,7 @@ int et_render_wavefront(et_scene* s, int n_frames, int first_frame, int W, int H
       A.box.scale[k] = ext > 0.0f ? 64.0f / ext : 0.0f;
     }
   }
-  const int grid_shade = nsm * 8;
+    const int grid_shade = nsm * 16;
   for (int f0 = 0; f0 < n_frames; f0 += frames_per_batch) {
     const int nf = std::min(frames_per_batch, n_frames - f0);
     for (int s0 = 0; s0 < spp; s0 += samples_per_batch) {
@@ -450,7 +486,7 @@ int et_render_wavefront(et_scene* s, int n_frames, int first_frame, int W, int H
       bt.f0 = f0; bt.nf = nf; bt.s0 = s0; bt.ns = std::min(samples_per_batch, spp - s0);
       bt.paths = (int64_t)nf * bt.ns * npix;
       A.bt = bt;
-      ET_CHECK_CUDA(cudaMemsetAsync(A.ctr, 0, sizeof(uint32_t) * C_N, stream));
+      ET_CHECK_CUDA(cudaMemsetAsync(A.ctr, 0, sizeof(uint32_t) * kCtrWords, stream));
       size_t pe = 0;   // profiling marks (et_render_profile; no-ops when off)
       ET_TRY(prof_begin(s, kProfRaygen, stream, &pe));
       wf_raygen<<<(unsigned)((bt.paths + 255) / 256), 256, 0, stream>>>(A);
@@ -459,8 +495,6 @@ int et_render_wavefront(et_scene* s, int n_frames, int first_frame, int W, int H
       int cur = 0;
       for (int b = 1; b <= max_depth; ++b) {
         const int nxt = cur ^ 1;
-        ET_CHECK_CUDA(cudaMemsetAsync(A.ctr + C_NRAY0 + nxt, 0, sizeof(uint32_t), stream));
-        ET_CHECK_CUDA(cudaMemsetAsync(A.ctr + C_NSH, 0, sizeof(uint32_t) * 3, stream));
         const bool sort_next = sorted && b < max_depth;
         Args At = A, Ash = A;
         At.perm = sorted && b > 1 ? sperm : nullptr;
@@ -472,7 +506,7 @@ int et_render_wavefront(et_scene* s, int n_frames, int first_frame, int W, int H
         ET_TRY(prof_begin(s, kProfTrace, stream, &pe));
         wf_trace<false><<<grid_c, 128, 0, stream>>>(At, cur, b);
         ET_CHECK_LAUNCH();
-        ET_TRY(prof_end(s, kProfTrace, pe, 0, A.ctr + C_NRAY0 + cur, stream));
+        ET_TRY(prof_end(s, kProfTrace, pe, 0, A.ctr + ctr_of(b, C_NRAY), stream));
         ET_TRY(prof_begin(s, kProfShade, stream, &pe));
         wf_shade<<<grid_shade, 256, 0, stream>>>(Ash, cur, b);
         ET_CHECK_LAUNCH();
@@ -483,12 +517,12 @@ int et_render_wavefront(et_scene* s, int n_frames, int first_frame, int W, int H
           ET_CHECK_CUDA(cub::DeviceRadixSort::SortPairs(stmp, stmp_bytes, skey, skey_alt, sval, sperm,
                                                         (int)bt.paths, 0, kSortBits, stream));
         }
-        ET_TRY(prof_end(s, kProfShade, pe, 0, A.ctr + C_NRAY0 + cur, stream));
+        ET_TRY(prof_end(s, kProfShade, pe, 0, A.ctr + ctr_of(b, C_NRAY), stream));
         if (s->dev.n_lights > 0 && b < max_depth) {
           ET_TRY(prof_begin(s, kProfShadow, stream, &pe));
           wf_trace<true><<<grid_s, 128, 0, stream>>>(A, cur, b);
           ET_CHECK_LAUNCH();
-          ET_TRY(prof_end(s, kProfShadow, pe, 0, A.ctr + C_NSH, stream));
+          ET_TRY(prof_end(s, kProfShadow, pe, 0, A.ctr + ctr_of(b, C_NSH), stream));
         }
         cur = nxt;
       }
