@@ -34,12 +34,18 @@
 // MMA waits are bounded (et_set_wait_budget); on expiry the kernel writes NaN
 // to the outputs it has not finished (the loss then reports it), waits a
 // second bounded time for its MMAs in flight and frees its TMEM.
+//
+// With C = 16 channels a pixel-step is one 64-byte row, and both kernels have a
+// second form (tct_conv16, tct_wgrad16) that moves whole tiles by TMA and keeps
+// its CTAs resident over many tiles; the forms above serve C < 16.
 #include "et_internal.cuh"
 #include "evsnet_common.h"
 #include "tc_ptx.cuh"
 #include "train_api.h"
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <algorithm>
+#include <cstring>
 
 namespace {
 
@@ -356,9 +362,524 @@ tct_wgrad(const float* __restrict__ dz, const float* __restrict__ in, int B, int
   if (warp == 0) tmem_dealloc(tmem, 32);
 }
 
+
+// ================================================================ C = 16, by TMA
+// Tensors are [B K][hw][16] FP32.  A box is one step of 128 pixels: 128 rows of
+// 64 bytes, 64-byte swizzled in shared memory, so that the 8 lanes of a 16-byte
+// access phase, each reading its own pixel's row, meet 32 different banks
+// (thread-per-pixel reads of global rows cost 16 lines per 512 bytes and left
+// the kernels at 28 % of the HBM rate).  Rows beyond hw are zero-filled on loads
+// and dropped on stores by the tensor map.
+constexpr int kBox = TP * CP * 4;       // bytes of one step's tile
+
+__device__ __forceinline__ const float4* box_row(const unsigned char* box, int p, int j) {
+  return reinterpret_cast<const float4*>(box + p * 64 + 16 * (j ^ ((p >> 1) & 3)));
+}
+__device__ __forceinline__ void box_load(const unsigned char* box, int p, float (&v)[CP]) {
+#pragma unroll
+  for (int j = 0; j < CP / 4; ++j) {
+    const float4 x = *box_row(box, p, j);
+    v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
+  }
+}
+__device__ __forceinline__ void box_store(unsigned char* box, int p, const float (&v)[CP]) {
+#pragma unroll
+  for (int j = 0; j < CP / 4; ++j)
+    *reinterpret_cast<float4*>(box + p * 64 + 16 * (j ^ ((p >> 1) & 3))) =
+        make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+}
+// shared memory -> the tensor's box at (x, y, z); completes with the issuing
+// thread's bulk group
+__device__ __forceinline__ void tma_store_3d(const void* tmap, int x, int y, int z, const void* src) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                   reinterpret_cast<uint64_t>(tmap)),
+               "r"(x), "r"(y), "r"(z), "r"(smem_u32(src))
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// every committed store has read its shared memory / has completed
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+struct Conv16Args {
+  int K, kt;
+  int64_t hw;
+  int tiles, nch;        // 128-pixel tiles per step; chunks of two steps per clip
+  int64_t total;         // B * tiles * nch chunks
+  const float* w;
+  const float* b;
+  int has_extra;
+  const float* wp;
+  const float* bp;
+  float* I;
+  uint32_t wait_iters;
+};
+
+// Same arithmetic as tct_conv, bit for bit.  Bound by HBM: per pixel-step 64
+// bytes of input and output each, plus the residual (forward) or the mask and
+// the added gradient (data gradient).  The B tiles nch chunks (a chunk = two
+// steps of a tile) are numbered with time innermost and split evenly over the
+// resident CTAs (2 per SM), so no last wave is half empty; a CTA that starts in
+// the middle of a clip first refills the ring with the kt - 1 steps before.
+// Shared memory per CTA: the ring (32 KB), the weights, and boxes: input x 2
+// (forward; 1 for the data gradient), O x 2 -- the residual or the mask, which
+// each thread overwrites with its own output row, stored from there by TMA --
+// and E, the data gradient's added term.  Thread 0 issues copies and MMAs: the
+// input box is requested again as soon as it is converted, an O box a whole
+// chunk ahead, once the store before has read it.
+template <bool kBwd>
+__global__ void __launch_bounds__(TP, 2)
+tct_conv16(const __grid_constant__ CUtensorMap m_in, const __grid_constant__ CUtensorMap m_extra,
+           const __grid_constant__ CUtensorMap m_mask, const __grid_constant__ CUtensorMap m_out, Conv16Args A) {
+  constexpr int kIn = kBwd ? 1 : 2;      // input chunk buffers
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ uint64_t in_bar[kIn], o_bar[2], e_bar, mma_bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ float sb[CP], swp[CP];
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int K = A.K, kt = A.kt, R = kt + 1, nch = A.nch;
+  unsigned char* in_box = sm;                                  // [kIn][2 steps]
+  unsigned char* o_box = in_box + kIn * 2 * kBox;              // [2][2 steps]
+  unsigned char* e_box = o_box + 2 * 2 * kBox;                 // [2 steps], data gradient only
+  unsigned char* ring = e_box + (kBwd ? 2 * kBox : 0);         // [R] slots
+  unsigned char* wB = ring + (size_t)R * kSlot;
+  // B strip as in tct_conv; the weights are read in their own order
+  for (int i = tid; i < kt * CP * CP; i += TP) {
+    const int tau = i % kt, r = i / kt, lo = r % CP, hi = r / CP;   // w[hi][lo][tau]
+    const int n = kBwd ? lo : hi, k = kBwd ? hi : lo;
+    unsigned char* dst = wB + (k >> 3) * (kt * CP * 16) + ((kt - 1 - tau) * CP + n) * 16 + (k & 7) * 2;
+    *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(A.w[i]);
+  }
+  if (tid < CP) {
+    sb[tid] = (!kBwd && A.b) ? A.b[tid] : 0.0f;
+    swp[tid] = (!kBwd && A.wp) ? A.wp[tid] : 0.0f;
+  }
+  if (warp == 0) tmem_alloc(&tmem_slot, 32);
+  if (tid == 0) {
+    for (int i = 0; i < kIn; ++i) mbar_init(&in_bar[i], 1);
+    mbar_init(&o_bar[0], 1);
+    mbar_init(&o_bar[1], 1);
+    mbar_init(&e_bar, 1);
+    mbar_init(&mma_bar, 1);
+  }
+  fence_proxy_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+  const uint32_t idesc16 = umma_idesc_bf16(TP, CP), idesc32 = umma_idesc_bf16(TP, 2 * CP);
+  const uint64_t a_desc0 = umma_desc(smem_u32(ring), kPlane, 128);
+  const uint64_t b_desc0 = umma_desc(smem_u32(wB), kt * CP * 16, 128);
+  constexpr uint64_t kBlock = (CP * 16) >> 4;
+  const float bpv = (!kBwd && A.bp) ? A.bp[0] : 0.0f;
+  const bool has_o = kBwd || A.has_extra != 0, has_e = kBwd && A.has_extra != 0;
+
+  // this CTA's chunks [t0, t1), preceded by the chunks that only refill the ring
+  const int64_t t0 = A.total * blockIdx.x / gridDim.x, t1 = A.total * (blockIdx.x + 1) / gridDim.x;
+  const int64_t ts = t0 - min((int64_t)(kt / 2), t0 % nch);
+  // processing order u = 0 .. K-1 is time s = u (forward) or s = K-1-u (data gradient)
+  auto step_of = [&](int u) { return kBwd ? K - 1 - u : u; };
+  // boxes of chunk t of a tensor (thread 0): coordinates (channel, pixel, clip step)
+  auto load_boxes = [&](const CUtensorMap* m, int64_t t, unsigned char* dst, uint64_t* bar) {
+    const int64_t seg = t / nch;
+    const int c = (int)(t - seg * nch), tile = (int)(seg % A.tiles), bc = (int)(seg / A.tiles);
+    const int n = min(2, K - 2 * c);
+    mbar_arrive_expect_tx(bar, (uint32_t)(n * kBox));
+    for (int j = 0; j < n; ++j)
+      tma_load_3d(dst + j * kBox, m, 0, tile * TP, bc * K + step_of(2 * c + j), bar);
+  };
+  uint32_t n_in[2] = {0, 0}, n_o[2] = {0, 0}, n_e = 0;   // thread 0: boxes requested per buffer
+  if (tid == 0 && ts < t1) {
+    for (int i = 0; i < kIn; ++i)
+      if (ts + i < t1) { load_boxes(&m_in, ts + i, in_box + i * 2 * kBox, &in_bar[i]); ++n_in[i]; }
+    if (has_o) { load_boxes(kBwd ? &m_mask : &m_extra, t0, o_box, &o_bar[0]); ++n_o[0]; }
+    if (has_e) { load_boxes(&m_extra, t0, e_box, &e_bar); ++n_e; }
+  }
+  uint32_t in_phase = 0, o_phase = 0, e_phase = 0, mma_phase = 0;   // next parities, one bit per buffer
+  int64_t seg = ts / nch;
+  int c = (int)(ts - seg * nch), tile = (int)(seg % A.tiles), bc = (int)(seg / A.tiles);
+  bool fresh = true;                     // the ring must be zero before this chunk
+  bool bail = false;
+  int n_mma = 0;
+  int64_t t = ts;
+  for (; t < t1; ++t) {
+    const int u0 = 2 * c, tc = min(2, K - u0);
+    const int64_t p = (int64_t)tile * TP + tid;
+    const bool live = p < A.hw;
+    bool fail = false;
+    if (fresh || c == 0) {
+      for (int i = tid; i < R * kSlot / 16; i += TP) reinterpret_cast<uint4*>(ring)[i] = make_uint4(0, 0, 0, 0);
+      __syncthreads();                   // a row of the ring is zeroed by one thread and filled by another
+      fresh = false;
+    }
+    // ---- the chunk's input, rounded to BF16, into the ring
+    {
+      const int bi = kIn == 1 ? 0 : (int)((t - ts) & 1);
+      fail |= !mbar_wait(&in_bar[bi], (in_phase >> bi) & 1u, A.wait_iters);
+      in_phase ^= 1u << bi;
+      for (int j = 0; j < tc; ++j) {
+        float v[CP];
+        box_load(in_box + (bi * 2 + j) * kBox, tid, v);
+        store_slot(ring + (size_t)((u0 + j) % R) * kSlot, tid, v);
+      }
+      fence_proxy_async_smem();
+      tc_fence_before();
+      bail = __syncthreads_or(fail) != 0;
+      if (bail) break;
+      tc_fence_after();
+      if (tid == 0 && t + kIn < t1) {
+        load_boxes(&m_in, t + kIn, in_box + bi * 2 * kBox, &in_bar[bi]);
+        ++n_in[bi];
+      }
+    }
+    if (t >= t0) {
+      const int oi = (int)((t - t0) & 1);
+      if (tid == 0) {
+        const int p0 = ((u0 - (kt - 1)) % R + R) % R;
+        auto a_of = [&](int i) {
+          const int pos = p0 + i >= R ? p0 + i - R : p0 + i;
+          return a_desc0 + (uint64_t)pos * (kSlot >> 4);
+        };
+        umma_bf16(tmem, a_of(0), b_desc0 + (uint64_t)(kt - 1) * kBlock, idesc16, 0);
+        if (tc > 1) umma_bf16(tmem + CP, a_of(kt), b_desc0, idesc16, 0);
+        for (int i = 1; i < kt; ++i)
+          umma_bf16(tmem, a_of(i), b_desc0 + (uint64_t)(kt - 1 - i) * kBlock, idesc32, 1);
+        umma_commit(&mma_bar);
+        // the other O buffer is free once the previous chunk's store has read it
+        bulk_wait_read();
+        if (has_o && t + 1 < t1) {
+          load_boxes(kBwd ? &m_mask : &m_extra, t + 1, o_box + (oi ^ 1) * 2 * kBox, &o_bar[oi ^ 1]);
+          ++n_o[oi ^ 1];
+        }
+      }
+      ++n_mma;
+      if (has_o) {
+        fail |= !mbar_wait(&o_bar[oi], (o_phase >> oi) & 1u, A.wait_iters);
+        o_phase ^= 1u << oi;
+      }
+      if (has_e) {
+        fail |= !mbar_wait(&e_bar, e_phase, A.wait_iters);
+        e_phase ^= 1u;
+      }
+      fail |= !mbar_wait(&mma_bar, mma_phase, A.wait_iters);
+      mma_phase ^= 1u;
+      // without a load into O, the store of two chunks ago must have read it
+      // (thread 0 waited for every store before it issued this chunk's MMAs,
+      // whose commit this thread has just seen)
+      tc_fence_after();
+      float acc[2][CP];
+      tmem_ld32(tmem + lane_base, &acc[0][0]);
+      for (int j = 0; j < tc; ++j) {
+        float ex[CP], mk[CP];
+        if (has_o) box_load(o_box + (oi * 2 + j) * kBox, tid, kBwd ? mk : ex);
+        if (has_e) box_load(e_box + j * kBox, tid, ex);
+        float v[CP];
+        float Iv = bpv;
+#pragma unroll
+        for (int co = 0; co < CP; ++co) {
+          if (!kBwd) {
+            float z = acc[j][co] + sb[co];
+            if (has_o) z += ex[co];
+            v[co] = fmaxf(z, 0.0f);
+            Iv = fmaf(swp[co], v[co], Iv);
+          } else {
+            float z = acc[j][co];
+            if (has_e) z += ex[co];
+            v[co] = mk[co] > 0.0f ? z : 0.0f;
+          }
+        }
+        box_store(o_box + (oi * 2 + j) * kBox, tid, v);
+        if (!kBwd && A.I && live) A.I[((int64_t)bc * K + step_of(u0 + j)) * A.hw + p] = Iv;
+      }
+      fence_proxy_async_smem();
+      tc_fence_before();
+      bail = __syncthreads_or(fail) != 0;
+      if (bail) break;
+      if (tid == 0) {
+        for (int j = 0; j < tc; ++j)
+          tma_store_3d(&m_out, 0, tile * TP, bc * K + step_of(u0 + j), o_box + (oi * 2 + j) * kBox);
+        bulk_commit();
+        if (has_e && t + 1 < t1) { load_boxes(&m_extra, t + 1, e_box, &e_bar); ++n_e; }
+      }
+    }
+    if (++c == nch) {
+      c = 0;
+      if (++tile == A.tiles) { tile = 0; ++bc; }
+    }
+  }
+  if (tid == 0) bulk_wait_all();
+  if (bail) {
+    // unfinished chunks: NaN (through the output's tensor map, like every
+    // store), so that the loss shows the failure; then the copies and MMAs in
+    // flight are waited for (bounded)
+    __syncthreads();
+    if (tid == 0) {
+      for (int i = 0; i < kIn; ++i)
+        if (n_in[i]) mbar_wait(&in_bar[i], (n_in[i] - 1) & 1u, kDrainIters);
+      for (int i = 0; i < 2; ++i)
+        if (n_o[i]) mbar_wait(&o_bar[i], (n_o[i] - 1) & 1u, kDrainIters);
+      if (n_e) mbar_wait(&e_bar, (n_e - 1) & 1u, kDrainIters);
+    }
+    if (n_mma) mbar_wait(&mma_bar, (uint32_t)(n_mma - 1) & 1u, kDrainIters);
+    __syncthreads();
+    float nan[CP];
+#pragma unroll
+    for (int i = 0; i < CP; ++i) nan[i] = __int_as_float(0x7fc00000);
+    box_store(o_box, tid, nan);
+    fence_proxy_async_smem();
+    __syncthreads();
+    for (t = max(t, t0); t < t1; ++t) {
+      const int64_t sg = t / nch;
+      const int ct = (int)(t - sg * nch), tl = (int)(sg % A.tiles), b = (int)(sg / A.tiles);
+      for (int u = 2 * ct; u < min(K, 2 * ct + 2); ++u) {
+        const int64_t row = (int64_t)b * K + step_of(u);
+        if (tid == 0) tma_store_3d(&m_out, 0, tl * TP, (int)row, o_box);
+        const int64_t p = (int64_t)tl * TP + tid;
+        if (!kBwd && A.I && p < A.hw) A.I[row * A.hw + p] = nan[0];
+      }
+    }
+    if (tid == 0) { bulk_commit(); bulk_wait_all(); }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tmem_dealloc(tmem, 32);
+}
+
+// Weight gradient, as tct_wgrad but without transposing: both operands are
+// MN-major, so a ring slot is the BF16 rows as they come (8-channel planes of
+// 128 pixels, 16-byte rows: a core matrix is 8 pixels of 8 channels), two
+// 16-byte stores per pixel and step instead of 32 two-byte ones.  A chunk of
+// two steps k, k + 1 meets the whole ring of 8 slots (steps k - 6 .. k + 1) in
+// 8 MMAs of M = 128 (slot, input channel), N = 32 (step, output channel),
+// K = 16 pixels; slot r and step j pair at tap (r - k - j + kt - 1) mod 8, no
+// tap where that is >= kt.  k mod 8 takes four values, so four accumulators of
+// 32 TMEM columns, each always for one of them, leave the tap of every entry
+// fixed while the ring turns.  The chunks are split evenly over the resident
+// CTAs (2 per SM) as in tct_conv16; an accumulator sums a quarter of its CTA's
+// chunks, one atomic per entry and CTA follows.  Bound by HBM: 128 bytes per
+// pixel-step (8 clips x 64 x 128 x 128: 0.50 ms transposed, 0.27 with one step
+// and N = 16 per 8 MMAs on a doubled ring, now 0.182; floor 0.158).
+constexpr int kWStage = 2;               // chunks in flight
+constexpr int kWAcc = 4;
+
+struct Wgrad16Args {
+  int K, kt;
+  int64_t hw;
+  int tiles, nch;
+  int64_t total;        // B * tiles * nch chunks
+  float* gw;
+  float* gb;
+  uint32_t wait_iters;
+};
+
+// kind::f16 instruction descriptor with both operands MN-major
+__host__ __device__ constexpr uint32_t umma_idesc_bf16_mn(int M, int N) {
+  return umma_idesc_bf16(M, N) | (1u << 15) | (1u << 16);
+}
+
+__global__ void __launch_bounds__(TP, 2)
+tct_wgrad16(const __grid_constant__ CUtensorMap m_dz, const __grid_constant__ CUtensorMap m_in, Wgrad16Args A) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ uint64_t bar[kWStage], mma_bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ float red[TP / 32][CP];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int K = A.K, kt = A.kt, nch = A.nch;
+  unsigned char* stage = sm;                                    // [kWStage][input x 2, dz x 2]
+  unsigned char* ring = stage + kWStage * 4 * kBox;             // [8] slots, step s at s mod 8
+  unsigned char* dslot = ring + 8 * kSlot;                      // [2]
+  if (warp == 0) tmem_alloc(&tmem_slot, kWAcc * 2 * CP);
+  if (tid == 0) {
+    for (int i = 0; i < kWStage; ++i) mbar_init(&bar[i], 1);
+    mbar_init(&mma_bar, 1);
+  }
+  fence_proxy_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+  const uint32_t idesc = umma_idesc_bf16_mn(TP, 2 * CP);
+  // MN-major, no swizzle: leading offset = next 8 pixels (K), stride offset =
+  // next 8 channels (the planes of consecutive slots are 2 KB apart)
+  const uint64_t a_desc = umma_desc(smem_u32(ring), 128, kPlane), b_desc = umma_desc(smem_u32(dslot), 128, kPlane);
+  const int64_t t0 = A.total * blockIdx.x / gridDim.x, t1 = A.total * (blockIdx.x + 1) / gridDim.x;
+  const int64_t ts = t0 - min((int64_t)(kt / 2), t0 % nch);
+  auto load_chunk = [&](int64_t t) {
+    const int64_t sg = t / nch;
+    const int k = 2 * (int)(t - sg * nch), tl = (int)(sg % A.tiles), b = (int)(sg / A.tiles), n = min(2, K - k);
+    const int i = (int)((t - ts) % kWStage);
+    unsigned char* dst = stage + i * 4 * kBox;
+    mbar_arrive_expect_tx(&bar[i], (uint32_t)(2 * n * kBox));
+    for (int j = 0; j < n; ++j) {
+      tma_load_3d(dst + j * kBox, &m_in, 0, tl * TP, b * K + k + j, &bar[i]);
+      tma_load_3d(dst + (2 + j) * kBox, &m_dz, 0, tl * TP, b * K + k + j, &bar[i]);
+    }
+  };
+  int64_t loaded = 0;                    // thread 0: chunks requested
+  if (tid == 0)
+    for (int i = 0; i < kWStage && ts + i < t1; ++i) { load_chunk(ts + i); ++loaded; }
+  float gbr[CP];
+#pragma unroll
+  for (int i = 0; i < CP; ++i) gbr[i] = 0.0f;
+  uint32_t phase = 0, mma_phase = 0;
+  uint32_t used = 0;                     // accumulators that hold something
+  int c = (int)(ts % nch);
+  bool fresh = true, bail = false;
+  int n_mma = 0;
+  for (int64_t t = ts; t < t1; ++t) {
+    const int si = (int)((t - ts) % kWStage), k = 2 * c, n = min(2, K - k);
+    bool fail = !mbar_wait(&bar[si], (phase >> si) & 1u, A.wait_iters);
+    phase ^= 1u << si;
+    // the previous chunk's MMAs have read the ring and the dz slots
+    if (n_mma) {
+      fail |= !mbar_wait(&mma_bar, mma_phase ^ 1u, A.wait_iters);
+      tc_fence_after();
+    }
+    if (fresh || c == 0) {
+      for (int i = tid; i < 8 * kSlot / 16; i += TP) reinterpret_cast<uint4*>(ring)[i] = make_uint4(0, 0, 0, 0);
+      __syncthreads();                   // a row of the ring is zeroed by one thread and filled by another
+      fresh = false;
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      float x[CP], d[CP];
+      if (j < n) {
+        box_load(stage + (si * 4 + j) * kBox, tid, x);
+        box_load(stage + (si * 4 + 2 + j) * kBox, tid, d);
+      } else {                           // no second step: zeros on both sides of its products
+#pragma unroll
+        for (int i = 0; i < CP; ++i) x[i] = d[i] = 0.0f;
+      }
+      store_slot(ring + ((k + j) & 7) * kSlot, tid, x);
+      store_slot(dslot + j * kSlot, tid, d);
+      if (t >= t0)
+#pragma unroll
+        for (int i = 0; i < CP; ++i) gbr[i] += d[i];
+    }
+    fence_proxy_async_smem();
+    tc_fence_before();
+    bail = __syncthreads_or(fail) != 0;
+    if (bail) break;
+    tc_fence_after();
+    if (tid == 0 && t + kWStage < t1) { load_chunk(t + kWStage); ++loaded; }
+    if (t >= t0) {
+      const int q = c & (kWAcc - 1);
+      if (tid == 0) {
+        for (int j = 0; j < TP / 16; ++j)
+          umma_bf16(tmem + (uint32_t)(q * 2 * CP), a_desc + (uint64_t)(j * 16), b_desc + (uint64_t)(j * 16), idesc,
+                    (((used >> q) & 1u) || j > 0) ? 1u : 0u);
+        umma_commit(&mma_bar);
+      }
+      used |= 1u << q;
+      ++n_mma;
+      mma_phase ^= 1u;
+    }
+    if (++c == nch) c = 0;
+  }
+  if (!bail && n_mma) {
+    const bool fail = !mbar_wait(&mma_bar, mma_phase ^ 1u, A.wait_iters);
+    bail = __syncthreads_or(fail) != 0;
+    tc_fence_after();
+  }
+  if (bail) {
+    if (tid == 0) {
+      for (int i = 0; i < kWStage; ++i) {
+        // requests so far into stage i: those numbered i, i + kWStage, ...
+        const int64_t m = (loaded - i + kWStage - 1) / kWStage;
+        if (m > 0) mbar_wait(&bar[i], (uint32_t)((m - 1) & 1), kDrainIters);
+      }
+      atomicAdd(A.gw, __int_as_float(0x7fc00000));   // the gradient reports the failure
+    }
+    if (n_mma) mbar_wait(&mma_bar, mma_phase ^ 1u, kDrainIters);
+  } else {
+    // the accumulators' entries summed per (tap, output, input channel) in the
+    // staging area (free: every chunk has been read)
+    float* sum = reinterpret_cast<float*>(stage);
+    for (int i = tid; i < kt * CP * CP; i += TP) sum[i] = 0.0f;
+    __syncthreads();
+    const int r = tid / CP, ci = tid % CP;   // lane = row (slot r, input channel ci)
+    for (int q = 0; q < kWAcc; ++q) {
+      if (!((used >> q) & 1u)) continue;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        float v[CP];
+        tmem_ld16(tmem + lane_base + (uint32_t)((2 * q + j) * CP), v);
+        const int tau = (r - 2 * q - j + kt - 1) & 7;
+        if (tau < kt)
+#pragma unroll
+          for (int co = 0; co < CP; ++co) atomicAdd(&sum[(tau * CP + co) * CP + ci], v[co]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < CP; ++i) {
+      float v = gbr[i];                  // rows beyond hw are zero
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+      if (lane == 0) red[warp][i] = v;
+    }
+    __syncthreads();
+    for (int i = tid; i < kt * CP * CP; i += TP) {   // gw[co][ci][tau]
+      const int tau = i % kt, cc = i / kt % CP, co = i / (kt * CP);
+      atomicAdd(A.gw + i, sum[(tau * CP + co) * CP + cc]);
+    }
+    if (tid < CP) {
+      float v = 0.0f;
+      for (int wv = 0; wv < TP / 32; ++wv) v += red[wv][tid];
+      atomicAdd(A.gb + tid, v);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tmem_dealloc(tmem, kWAcc * 2 * CP);
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- host
+namespace {
+
+// tensor map of [steps][hw][16] floats, box = one step of 128 pixels
+int map_rows(CUtensorMap* m, const float* base, int64_t steps, int64_t hw) {
+  typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static const EncodeFn encode = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult qr;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &qr) !=
+            cudaSuccess || qr != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return reinterpret_cast<EncodeFn>(f);
+  }();
+  if (!encode) return ET_ERR_CUDA;
+  const cuuint64_t dims[3] = {(cuuint64_t)CP, (cuuint64_t)hw, (cuuint64_t)steps};
+  const cuuint64_t strides[2] = {(cuuint64_t)CP * 4, (cuuint64_t)hw * CP * 4};
+  const cuuint32_t box[3] = {(cuuint32_t)CP, (cuuint32_t)TP, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS ? ET_OK : ET_ERR_CUDA;
+}
+
+// the TMA forms: 16 channels, 16-byte aligned tensors, coordinates within 31 bits
+bool use_tma(int B, int K, int64_t hw, int C, const float* a, const float* b) {
+  return C == CP && (int64_t)B * K < (1ll << 31) && hw < (1ll << 31) - TP &&
+         ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+}
+
+int resident_ctas(int64_t work, int* out) {
+  int dev = 0, nsm = 0;
+  ET_CHECK_CUDA(cudaGetDevice(&dev));
+  ET_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  *out = (int)std::max<int64_t>(1, std::min<int64_t>(work, 2 * nsm));
+  return ET_OK;
+}
+
+}  // namespace
+
 bool et_train_tct_supported(const et_evsnet_weights* net) {
   return net->kt >= 1 && net->kt <= kMaxKtTc && net->C >= 1 && net->C <= CP;
 }
@@ -367,6 +888,29 @@ int et_train_tct_conv(const float* in, int B, int K, int64_t hw, int C, int kt, 
                       const float* extra, const float* mask, float* out, const float* wp, const float* bp,
                       float* I, bool data_grad, cudaStream_t st) {
   if (kt < 1 || kt > kMaxKtTc || C < 1 || C > CP || B < 1 || K < 1 || hw < 1) return ET_ERR_UNIMPLEMENTED;
+  if (use_tma(B, K, hw, C, in, out) && use_tma(B, K, hw, C, extra, mask)) {
+    const int64_t tiles = (hw + TP - 1) / TP, nch = (K + 1) / 2;
+    Conv16Args A{K, kt, hw, (int)tiles, (int)nch, B * tiles * nch, w, b, extra != nullptr, wp, bp, I,
+                 et_tc_wait_iters()};
+    CUtensorMap m_in, m_extra, m_mask, m_out;
+    std::memset(&m_extra, 0, sizeof(m_extra));
+    std::memset(&m_mask, 0, sizeof(m_mask));
+    int rc = map_rows(&m_in, in, (int64_t)B * K, hw);
+    if (rc == ET_OK) rc = map_rows(&m_out, out, (int64_t)B * K, hw);
+    if (rc == ET_OK && extra) rc = map_rows(&m_extra, extra, (int64_t)B * K, hw);
+    if (rc == ET_OK && data_grad) rc = map_rows(&m_mask, mask, (int64_t)B * K, hw);
+    int grid = 0;
+    if (rc == ET_OK) rc = resident_ctas(A.total, &grid);
+    if (rc != ET_OK) return rc;
+    // input x 2 and O x 2 (forward), or input, O x 2 and E: four or four chunks
+    const size_t smem = (size_t)(data_grad ? 1 + 2 + 1 : 2 + 2) * 2 * kBox + (size_t)(kt + 1) * kSlot +
+                        (size_t)kt * CP * CP * 2;
+    auto kern = data_grad ? tct_conv16<true> : tct_conv16<false>;
+    ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<grid, TP, smem, st>>>(m_in, m_extra, m_mask, m_out, A);
+    ET_CHECK_LAUNCH();
+    return ET_OK;
+  }
   ConvArgs A{in, B, K, C, kt, hw, w, b, extra, mask, out, wp, bp, I, et_tc_wait_iters()};
   const size_t smem = (size_t)(kt + 1) * kSlot + (size_t)kt * CP * CP * 2;
   const int64_t blocks = (int64_t)B * ((hw + TP - 1) / TP);
@@ -384,6 +928,21 @@ int et_train_tct_conv(const float* in, int B, int K, int64_t hw, int C, int kt, 
 int et_train_tct_wgrad(const float* dz, const float* in, int B, int K, int64_t hw, int C, int kt, float* gw,
                        float* gb, cudaStream_t st) {
   if (kt < 1 || kt > kMaxKtTc || C < 1 || C > CP || B < 1 || K < 1 || hw < 1) return ET_ERR_UNIMPLEMENTED;
+  if (use_tma(B, K, hw, C, dz, in)) {
+    const int64_t tiles = (hw + TP - 1) / TP, nch = (K + 1) / 2;
+    Wgrad16Args A{K, kt, hw, (int)tiles, (int)nch, B * tiles * nch, gw, gb, et_tc_wait_iters()};
+    CUtensorMap m_dz, m_in;
+    int rc = map_rows(&m_dz, dz, (int64_t)B * K, hw);
+    if (rc == ET_OK) rc = map_rows(&m_in, in, (int64_t)B * K, hw);
+    int grid = 0;
+    if (rc == ET_OK) rc = resident_ctas(A.total, &grid);
+    if (rc != ET_OK) return rc;
+    const size_t smem = (size_t)kWStage * 4 * kBox + 10 * kSlot;
+    ET_CHECK_CUDA(cudaFuncSetAttribute(tct_wgrad16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    tct_wgrad16<<<grid, TP, smem, st>>>(m_dz, m_in, A);
+    ET_CHECK_LAUNCH();
+    return ET_OK;
+  }
   const size_t smem = (size_t)kWABytes + kWBBytes;
   const int64_t blocks = (int64_t)B * ((hw + TP - 1) / TP);
   if (blocks > 0x7FFFFFFF) return ET_ERR_ARG;
