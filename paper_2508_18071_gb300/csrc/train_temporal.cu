@@ -40,90 +40,209 @@ inline int layer0_taps(const et_evsnet_weights* net) {
 }
 
 // ------------------------------------------------------- forward conv, layer 0
-// One thread per (clip, step, pixel); X read as l_{k+1} - l_k from the clip's
-// log frames.  A one-layer network also writes the projection I = bp + wp . out.
-__global__ void __launch_bounds__(256, 4)
+// 64 bytes written per pixel-step.  One thread per pixel computes
+// all channels; a warp's 32 rows then go through shared memory (16-byte pieces
+// permuted so that neither side meets a bank twice) and leave as whole 512-byte
+// lines.  X is read as l_{k+1} - l_k from the clip's log frames.
+constexpr int kMaxStem = 7;
+
+// ReLU of a warp's 32 rows (lane = pixel idx0 + lane, `n` of them in the image)
+// to out; a one-layer network also writes the projection I = bp + wp . out.
+// stage: the warp's 2 KB.
+__device__ __forceinline__ void store_rows(float (&acc)[kMaxC], int64_t idx0, int n, int C, float* stage,
+                                           float* __restrict__ out, const float* __restrict__ wp,
+                                           const float* __restrict__ bp, float* __restrict__ I) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int c = 0; c < kMaxC; ++c) acc[c] = fmaxf(acc[c], 0.0f);
+  if (I && lane < n) {
+    float Iv = bp[0];
+#pragma unroll
+    for (int c = 0; c < kMaxC; ++c)
+      if (c < C) Iv = fmaf(wp[c], acc[c], Iv);
+    I[idx0 + lane] = Iv;
+  }
+  if (C == kMaxC) {
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      *reinterpret_cast<float4*>(stage + lane * kMaxC + 4 * (j ^ ((lane >> 1) & 3))) =
+          make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int pix = r * 8 + (lane >> 2), j = lane & 3;
+      const float4 v = *reinterpret_cast<const float4*>(stage + pix * kMaxC + 4 * (j ^ ((pix >> 1) & 3)));
+      if (pix < n) *reinterpret_cast<float4*>(out + (idx0 + pix) * kMaxC + 4 * j) = v;
+    }
+  } else if (lane < n) {
+#pragma unroll
+    for (int c = 0; c < kMaxC; ++c)
+      if (c < C) out[(idx0 + lane) * C + c] = acc[c];
+  }
+}
+
+__device__ __forceinline__ void fma_tap(const float* __restrict__ w, float x, float (&acc)[kMaxC]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float4 v = reinterpret_cast<const float4*>(w)[j];
+    acc[4 * j] = fmaf(v.x, x, acc[4 * j]);
+    acc[4 * j + 1] = fmaf(v.y, x, acc[4 * j + 1]);
+    acc[4 * j + 2] = fmaf(v.z, x, acc[4 * j + 2]);
+    acc[4 * j + 3] = fmaf(v.w, x, acc[4 * j + 3]);
+  }
+}
+
+// [tap][channel] and biases, zero beyond C
+__device__ __forceinline__ void stage_taps(float (*sw)[kMaxC], float* sb, const float* __restrict__ w,
+                                           const float* __restrict__ b, int taps, int C) {
+  for (int i = threadIdx.x; i < kMaxC * taps; i += blockDim.x) {
+    const int t = i / kMaxC, c = i % kMaxC;
+    sw[t][c] = c < C ? w[c * taps + t] : 0.0f;
+  }
+  if (threadIdx.x < kMaxC) sb[threadIdx.x] = threadIdx.x < C ? b[threadIdx.x] : 0.0f;
+  __syncthreads();
+}
+
+// Temporal layer 0, taps over the last kt steps: a thread walks kWalk steps of
+// its pixel with the last T = 7 or 9 X in registers (T >= kt), one new log
+// value per step (4 clips x 64 x 128 x 128: 0.30 -> 0.062 ms; HBM floor 0.042).
+constexpr int kWalk = 16;
+template <int T>
+__global__ void __launch_bounds__(128)
 tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, int kt,
           const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
           const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
-  constexpr int Cin = 1;
-  __shared__ float sw[kMaxC * kMaxC * kMaxKt];
-  for (int i = threadIdx.x; i < C * Cin * kt; i += blockDim.x) sw[i] = w[i];
-  __syncthreads();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)B * K * hw) return;
-  const int64_t p = idx % hw;
-  const int k = (int)((idx / hw) % K), bc = (int)(idx / (hw * K));
-  float acc[kMaxC];
+  __shared__ __align__(16) float sw[kMaxKt][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
+  stage_taps(sw, sb, w, b, kt, C);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t groups = (uint32_t)((hw + 31) / 32), segs = (uint32_t)(K + kWalk - 1) / kWalk;
+  const uint32_t it = blockIdx.x * 4 + warp;
+  if (it >= (uint32_t)B * segs * groups) return;
+  const int64_t p0 = (int64_t)(it % groups) * 32, p = min(p0 + lane, hw - 1);
+  const int n = (int)min((int64_t)32, hw - p0);
+  const int k0 = (int)(it / groups % segs) * kWalk, bc = (int)(it / groups / segs);
+  const float* lf = logl + (int64_t)bc * (K + 1) * hw + p;
+  float xs[T];                            // X of steps k - T + 1 .. k
 #pragma unroll
-  for (int co = 0; co < kMaxC; ++co) acc[co] = co < C ? b[co] : 0.0f;
-  for (int tau = 0; tau < kt; ++tau) {
-    const int kk = k - (kt - 1) + tau;
-    if (kk < 0) continue;
-    const float* lf = logl + (int64_t)bc * (K + 1) * hw;
-    const float x = lf[(int64_t)(kk + 1) * hw + p] - lf[(int64_t)kk * hw + p];
-#pragma unroll
-    for (int co = 0; co < kMaxC; ++co)
-      if (co < C) acc[co] += sw[co * kt + tau] * x;
+  for (int t = 1; t < T; ++t) {
+    const int k = k0 - T + t;
+    xs[t] = k >= 0 ? lf[(int64_t)(k + 1) * hw] - lf[(int64_t)k * hw] : 0.0f;
   }
-  float* dst = out + idx * C;
-  float Iv = bp ? bp[0] : 0.0f;
+  float prev = lf[(int64_t)k0 * hw];
+  const int ns = min(kWalk, K - k0);
+  float nxt = lf[(int64_t)(k0 + 1) * hw];
+  for (int j = 0; j < ns; ++j) {
+    const int k = k0 + j;
 #pragma unroll
-  for (int co = 0; co < kMaxC; ++co) {
-    if (co >= C) break;
-    const float a = fmaxf(acc[co], 0.0f);
-    dst[co] = a;
-    if (I) Iv += wp[co] * a;
+    for (int t = 0; t + 1 < T; ++t) xs[t] = xs[t + 1];
+    xs[T - 1] = nxt - prev;
+    prev = nxt;
+    nxt = lf[(int64_t)min(k + 2, K) * hw];
+    float acc[kMaxC];
+#pragma unroll
+    for (int c = 0; c < kMaxC; ++c) acc[c] = sb[c];
+    const int tau0 = max(0, kt - 1 - k) + T - kt;   // steps before the clip are zero: no product
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+      if (t >= tau0) fma_tap(sw[t - (T - kt)], xs[t], acc);
+    store_rows(acc, ((int64_t)bc * K + k) * hw + p0, n, C, stage[warp], out, wp, bp, I);
   }
-  if (I) I[idx] = Iv;
 }
 
-// ------------------------------------------------- forward, spatial stem
-// Layer 0 as a one-step ks0 x ks0 convolution of X (zero outside the image);
-// one thread per (clip, step, pixel), taps in row-major order.
-constexpr int kMaxStem = 7;
-__global__ void __launch_bounds__(256, 4)
+// 3 x 3 spatial stem (one step, zero outside the image, taps in row-major
+// order): a thread walks kRows rows of one column of one step with the X of
+// three rows x three columns in registers (8 clips x 64 steps x 128 x 128: 0.50
+// ms with 4-byte pieces written 64 bytes apart, now 0.167; HBM floor 0.084).
+constexpr int kRows = 16;
+struct Rows3 {
+  const float* l1;                        // the step's frame and the one before, at the thread's column
+  const float* l0;
+  int H, W;
+  bool lft, rgt;
+  // X of row y, columns x - 1 .. x + 1, zero outside the image (loads always
+  // inside it, so that the next rows' loads need no branch)
+  __device__ __forceinline__ void load(int y, float (&r)[3]) const {
+    const bool in = y >= 0 && y < H;
+    const int64_t o = (int64_t)min(max(y, 0), H - 1) * W, ol = o - (lft ? 1 : 0), og = o + (rgt ? 1 : 0);
+    const float a = l1[ol] - l0[ol], b = l1[o] - l0[o], c = l1[og] - l0[og];
+    r[0] = in && lft ? a : 0.0f;
+    r[1] = in ? b : 0.0f;
+    r[2] = in && rgt ? c : 0.0f;
+  }
+};
+
+__global__ void __launch_bounds__(128)
+tstem3_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C,
+           const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
+           const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
+  __shared__ __align__(16) float sw[9][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
+  stage_taps(sw, sb, w, b, 9, C);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t hw = (int64_t)H * W;
+  const uint32_t groups = (uint32_t)(W + 31) / 32, strips = (uint32_t)(H + kRows - 1) / kRows;
+  const uint32_t it = blockIdx.x * 4 + warp;
+  if (it >= (uint32_t)B * K * strips * groups) return;
+  const int x0 = (int)(it % groups) * 32, x = min(x0 + lane, W - 1), y0 = (int)(it / groups % strips) * kRows;
+  const uint32_t bk = it / groups / strips;
+  const float* l1 = logl + ((int64_t)(bk / K) * (K + 1) + bk % K + 1) * hw + x;
+  const Rows3 R{l1, l1 - hw, H, W, x > 0, x + 1 < W};
+  float r0[3], r1[3], r2[3];
+  R.load(y0 - 1, r0);
+  R.load(y0, r1);
+  const int ny = min(kRows, H - y0);
+  R.load(y0 + 1, r2);
+  for (int j = 0; j < ny; ++j) {
+    const int y = y0 + j;
+    float nx[3];
+    R.load(y + 2, nx);
+    float acc[kMaxC];
+#pragma unroll
+    for (int c = 0; c < kMaxC; ++c) acc[c] = sb[c];
+    const bool up = y > 0, dn = y + 1 < H;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      const float v = t < 3 ? r0[t % 3] : t < 6 ? r1[t % 3] : r2[t % 3];
+      // taps outside the image: no product
+      if ((t >= 3 || up) && (t < 6 || dn) && (t % 3 != 0 || R.lft) && (t % 3 != 2 || R.rgt)) fma_tap(sw[t], v, acc);
+    }
+    store_rows(acc, (int64_t)bk * hw + (int64_t)y * W + x0, min(32, W - x0), C, stage[warp], out, wp, bp, I);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) { r0[t] = r1[t]; r1[t] = r2[t]; r2[t] = nx[t]; }
+  }
+}
+
+// the other stem sizes, one thread per pixel-step
+__global__ void __launch_bounds__(128)
 tstem_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C, int ks0,
           const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
           const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
-  __shared__ float sw[kMaxStem * kMaxStem][kMaxC];   // [tap][co]
-  for (int i = threadIdx.x; i < C * ks0 * ks0; i += blockDim.x) sw[i % (ks0 * ks0)][i / (ks0 * ks0)] = w[i];
-  __syncthreads();
+  __shared__ __align__(16) float sw[kMaxStem * kMaxStem][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
+  stage_taps(sw, sb, w, b, ks0 * ks0, C);
   const int64_t hw = (int64_t)H * W;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)B * K * hw) return;
-  const int64_t p = idx % hw;
-  const int k = (int)((idx / hw) % K), bc = (int)(idx / (hw * K));
-  const int y = (int)(p / W), x = (int)(p % W), r0 = ks0 >> 1;
-  const float* l1 = logl + ((int64_t)bc * (K + 1) + k + 1) * hw;
-  const float* l0 = l1 - hw;
-  float acc[kMaxC];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = ks0 >> 1;
+  const int64_t p0 = ((int64_t)blockIdx.x * 4 + warp) * 32, p = min(p0 + lane, hw - 1);
+  if (p0 >= hw) return;
+  const int y = (int)(p / W), x = (int)(p - (int64_t)y * W);
+  for (int bk = blockIdx.y; bk < B * K; bk += gridDim.y) {
+    const float* l1 = logl + ((int64_t)(bk / K) * (K + 1) + bk % K + 1) * hw;
+    const float* l0 = l1 - hw;
+    float acc[kMaxC];
 #pragma unroll
-  for (int co = 0; co < kMaxC; ++co) acc[co] = co < C ? b[co] : 0.0f;
-  for (int dy = 0; dy < ks0; ++dy) {
-    const int yy = y + dy - r0;
-    if (yy < 0 || yy >= H) continue;
-    for (int dx = 0; dx < ks0; ++dx) {
-      const int xx = x + dx - r0;
-      if (xx < 0 || xx >= W) continue;
-      const int64_t q = (int64_t)yy * W + xx;
-      const float v = l1[q] - l0[q];
-      const float* wt = sw[dy * ks0 + dx];
-#pragma unroll
-      for (int co = 0; co < kMaxC; ++co)
-        if (co < C) acc[co] = fmaf(wt[co], v, acc[co]);
+    for (int c = 0; c < kMaxC; ++c) acc[c] = sb[c];
+    for (int dy = 0; dy < ks0; ++dy) {
+      const int yy = y + dy - r0;
+      if (yy < 0 || yy >= H) continue;
+      for (int dx = 0; dx < ks0; ++dx) {
+        const int xx = x + dx - r0;
+        if (xx < 0 || xx >= W) continue;
+        const int64_t q = (int64_t)yy * W + xx;
+        fma_tap(sw[dy * ks0 + dx], l1[q] - l0[q], acc);
+      }
     }
+    __syncwarp();
+    store_rows(acc, (int64_t)bk * hw + p0, (int)min((int64_t)32, hw - p0), C, stage[warp], out, wp, bp, I);
   }
-  float* dst = out + idx * C;
-  float Iv = bp ? bp[0] : 0.0f;
-#pragma unroll
-  for (int co = 0; co < kMaxC; ++co) {
-    if (co >= C) break;
-    const float a = fmaxf(acc[co], 0.0f);
-    dst[co] = a;
-    if (I) Iv += wp[co] * a;
-  }
-  if (I) I[idx] = Iv;
 }
 
 // --------------------------------------------------------------------- BiLIF
@@ -189,110 +308,234 @@ __global__ void tbilif_bwd(const float* __restrict__ I, int B, int K, int64_t hw
 
 // ------------------------------------------------------ projection backward
 // dz[c] = dI wp[c] 1(h > 0); grad wp[c] += sum dI h[c]; grad bp += sum dI.
+// Bound by HBM (132 bytes per pixel-step): four lanes per pixel-step, 16-byte
+// accesses (8 clips x 64 steps x 128 x 128: 0.57 -> 0.19 ms).
+// a quad's channels 4 g .. of row idx (zero beyond C)
+__device__ __forceinline__ float4 load_quad(const float* __restrict__ src, int64_t idx, int g, int C) {
+  if (C == kMaxC) return __ldg(reinterpret_cast<const float4*>(src + idx * kMaxC) + g);
+  const float* r = src + idx * C + 4 * g;
+  return make_float4(4 * g < C ? r[0] : 0.0f, 4 * g + 1 < C ? r[1] : 0.0f, 4 * g + 2 < C ? r[2] : 0.0f,
+                     4 * g + 3 < C ? r[3] : 0.0f);
+}
+
 __global__ void __launch_bounds__(256)
 tproj_bwd(const float* __restrict__ dI, const float* __restrict__ h, int64_t n, int C,
           const float* __restrict__ wp, float* __restrict__ dz, float* __restrict__ gwp,
           float* __restrict__ gbp) {
-  __shared__ float red[kMaxC + 1][8];
-  float acc[kMaxC + 1];
+  __shared__ float red[8][kMaxC + 1];
+  const int g = threadIdx.x & 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float wv[4], acc[4] = {}, accd = 0.0f;
 #pragma unroll
-  for (int c = 0; c <= kMaxC; ++c) acc[c] = 0.0f;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  for (int j = 0; j < 4; ++j) wv[j] = 4 * g + j < C ? wp[4 * g + j] : 0.0f;
+#pragma unroll 4
+  for (int64_t i = (int64_t)blockIdx.x * 64 + (threadIdx.x >> 2); i < n; i += (int64_t)gridDim.x * 64) {
     const float d = dI[i];
-    acc[kMaxC] += d;
+    const float4 a = load_quad(h, i, g, C);
+    const float av[4] = {a.x, a.y, a.z, a.w};
+    float z[4];
+    accd += d;
 #pragma unroll
-    for (int c = 0; c < kMaxC; ++c) {
-      if (c >= C) break;
-      const float a = h[i * C + c];
-      acc[c] += d * a;
-      dz[i * C + c] = a > 0.0f ? d * wp[c] : 0.0f;
+    for (int j = 0; j < 4; ++j) {
+      acc[j] += d * av[j];
+      z[j] = av[j] > 0.0f ? d * wv[j] : 0.0f;
+    }
+    if (C == kMaxC) {
+      *reinterpret_cast<float4*>(dz + i * kMaxC + 4 * g) = make_float4(z[0], z[1], z[2], z[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (4 * g + j < C) dz[i * C + 4 * g + j] = z[j];
     }
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int c = 0; c <= kMaxC; ++c) {
-    float v = acc[c];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    if (lane == 0) red[c][warp] = v;
+  for (int o = 4; o < 32; o <<= 1) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] += __shfl_xor_sync(0xFFFFFFFFu, acc[j], o);
+    accd += __shfl_xor_sync(0xFFFFFFFFu, accd, o);
   }
+  if (lane < 4)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) red[warp][4 * g + j] = acc[j];
+  if (lane == 0) red[warp][kMaxC] = accd;
   __syncthreads();
   if (threadIdx.x < C || threadIdx.x == kMaxC) {
     float v = 0.0f;
-    for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) v += red[threadIdx.x][wv];
-    if (threadIdx.x < C) atomicAdd(gwp + threadIdx.x, v);
-    else atomicAdd(gbp, v);
+    for (int wr = 0; wr < 8; ++wr) v += red[wr][threadIdx.x];
+    atomicAdd(threadIdx.x < C ? gwp + threadIdx.x : gbp, v);
   }
 }
 
 // ------------------------------------------------- weight backward, layer 0
-// grad w[co][tau] += sum dz[k][co] X[k - kt + 1 + tau]; grad b[co] += sum dz[k][co].
-// Persistent blocks stage 128 pixel-steps at a time in shared memory; each
-// thread owns a (co, tau) entry, one atomic per entry per block.
-constexpr int kPts = 128;
-__global__ void __launch_bounds__(256)
-tconv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K,
-                 int64_t hw, int C, int kt, float* __restrict__ gw, float* __restrict__ gb) {
-  constexpr int Cin = 1;
-  __shared__ float sd[kPts][kMaxC];
-  __shared__ float sx[kPts][kMaxKt + 1];   // [tau], padded
-  constexpr int kPer = (kMaxC * kMaxKt + kMaxC + 255) / 256;
-  float acc[kPer];
+// Four lanes per pixel (lane g = output channels 4 g ..), the taps' sums in
+// registers; one atomic per entry per block at the end.
+// sums over the 8 pixels of a warp and the warps of a block, added to
+// gw[co * taps + t] and gb[co]
+template <int T>
+__device__ __forceinline__ void quad_grads(float (&acc)[T][4], float (&bias)[4], int g, int C, int taps, int t0,
+                                           float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ float red[T + 1][kMaxC];
+  for (int i = threadIdx.x; i < (T + 1) * kMaxC; i += blockDim.x) (&red[0][0])[i] = 0.0f;
+  __syncthreads();
 #pragma unroll
-  for (int j = 0; j < kPer; ++j) acc[j] = 0.0f;
-  const int nent = C * Cin * kt + C;
-  const int64_t npts = (int64_t)B * K * hw;
-  for (int64_t c0 = (int64_t)blockIdx.x * kPts; c0 < npts; c0 += (int64_t)gridDim.x * kPts) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < kPts * C; i += blockDim.x) {
-      const int pt = i / C, co = i % C;
-      const int64_t idx = c0 + pt;
-      sd[pt][co] = idx < npts ? dz[idx * C + co] : 0.0f;
-    }
-    for (int i = threadIdx.x; i < kPts * Cin * kt; i += blockDim.x) {
-      const int pt = i / (Cin * kt), r = i % (Cin * kt), ci = r / kt, tau = r % kt;
-      const int64_t idx = c0 + pt;
-      float v = 0.0f;
-      if (idx < npts) {
-        const int64_t p = idx % hw;
-        const int k = (int)((idx / hw) % K), bc = (int)(idx / (hw * K));
-        const int kk = k - (kt - 1) + tau;
-        if (kk >= 0) {
-          const float* lf = logl + (int64_t)bc * (K + 1) * hw;
-          v = lf[(int64_t)(kk + 1) * hw + p] - lf[(int64_t)kk * hw + p];
-        }
-      }
-      sx[pt][ci * kt + tau] = v;
-    }
-    __syncthreads();
+  for (int t = 0; t <= T; ++t)
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      const int e = threadIdx.x + j * 256;
-      if (e >= nent) break;
-      float s = 0.0f;
-      if (e < C * Cin * kt) {
-        const int co = e / (Cin * kt), r = e % (Cin * kt);
-        for (int pt = 0; pt < kPts; ++pt) s += sd[pt][co] * sx[pt][r];
-      } else {
-        const int co = e - C * Cin * kt;
-        for (int pt = 0; pt < kPts; ++pt) s += sd[pt][co];
-      }
-      acc[j] += s;
+    for (int j = 0; j < 4; ++j) {
+      float v = t < T ? acc[t < T ? t : 0][j] : bias[j];
+      for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+      if ((threadIdx.x & 31) < 4) atomicAdd(&red[t][4 * g + j], v);
     }
-  }
-#pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    const int e = threadIdx.x + j * 256;
-    if (e >= nent) break;
-    if (e < C * Cin * kt) atomicAdd(gw + e, acc[j]);
-    else atomicAdd(gb + (e - C * Cin * kt), acc[j]);
+  __syncthreads();
+  for (int i = threadIdx.x; i < (T + 1) * kMaxC; i += blockDim.x) {
+    const int t = i / kMaxC, co = i % kMaxC;
+    if (co >= C) continue;
+    if (t == T) atomicAdd(gb + co, red[t][co]);
+    else if (t >= t0) atomicAdd(gw + co * taps + t - t0, red[t][co]);
   }
 }
 
+// Rows of dz on their way to one lane (its own 16 bytes of each): kAhead rows in
+// flight by cp.async, since the taps' sums leave registers for 16 warps per SM
+// only and a warp's 512 bytes per row are far from covering the HBM latency.
+constexpr int kAhead = 8;
+struct QuadRing {
+  float4* slot;                            // this lane's first slot; the next one is 256 float4 on
+  const float* src;
+  int64_t idx0, step;                      // row of step j: idx0 + j step
+  int g, C, n;
+  __device__ __forceinline__ void request(int j) {
+    if (C == kMaxC && j < n)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(slot + (j & (kAhead - 1)) * 256)),
+                   "l"(src + (idx0 + j * step) * kMaxC + 4 * g)
+                   : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __device__ __forceinline__ void start() {
+#pragma unroll
+    for (int j = 0; j < kAhead - 1; ++j) request(j);
+  }
+  // row j (in order), requesting row j + kAhead - 1
+  __device__ __forceinline__ float4 take(int j) {
+    request(j + kAhead - 1);
+    if (C != kMaxC) return load_quad(src, idx0 + j * step, g, C);
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
+    return slot[(j & (kAhead - 1)) * 256];
+  }
+};
+
+// Temporal layer 0: grad w[co][tau] += sum dz[k][co] X[k - kt + 1 + tau];
+// grad b[co] += sum dz[k][co].  A thread walks kWalkB steps of one pixel with
+// the last T = 7 or 9 X in registers (T >= kt; the taps before are dropped):
+// one new log value and one 16-byte row piece per step.  68 bytes per pixel-step
+// (4 clips x 64 x 128 x 128: 0.41 ms with staged pixel-steps, 0.21 without the
+// row ring, now 0.112; HBM floor 0.042).
+constexpr int kWalkB = 32;
+template <int T>
+__global__ void __launch_bounds__(256, 2)
+tconv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K,
+                 int64_t hw, int C, int kt, float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ float4 ring[kAhead * 256];
+  const int g = threadIdx.x & 3, pl = (threadIdx.x & 31) >> 2;
+  float acc[T][4] = {}, bias[4] = {};
+  // (a clip batch that fits the device has fewer than 2^32 rows: 32-bit item numbers)
+  const uint32_t groups = (uint32_t)((hw + 7) / 8), segs = (uint32_t)(K + kWalkB - 1) / kWalkB;
+  const uint32_t items = (uint32_t)B * segs * groups;
+  for (uint32_t it = blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += gridDim.x * 8) {
+    const int64_t p = (int64_t)(it % groups) * 8 + pl;
+    const int k0 = (int)(it / groups % segs) * kWalkB, bc = (int)(it / groups / segs);
+    if (p >= hw) continue;
+    const int n = min(kWalkB, K - k0);
+    QuadRing rows{ring + threadIdx.x, dz, ((int64_t)bc * K + k0) * hw + p, hw, g, C, n};
+    rows.start();
+    const float* lf = logl + (int64_t)bc * (K + 1) * hw + p;
+    float xs[T];                          // X of steps k - T + 1 .. k
+#pragma unroll
+    for (int t = 1; t < T; ++t) {
+      const int k = k0 - T + t;
+      xs[t] = k >= 0 ? lf[(int64_t)(k + 1) * hw] - lf[(int64_t)k * hw] : 0.0f;
+    }
+    float prev = lf[(int64_t)k0 * hw], nxt[4];   // log values of the next four steps
+#pragma unroll
+    for (int t = 0; t < 4; ++t) nxt[t] = lf[(int64_t)min(k0 + 1 + t, K) * hw];
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+#pragma unroll
+      for (int t = 0; t + 1 < T; ++t) xs[t] = xs[t + 1];
+      xs[T - 1] = nxt[0] - prev;
+      prev = nxt[0];
+#pragma unroll
+      for (int t = 0; t < 3; ++t) nxt[t] = nxt[t + 1];
+      nxt[3] = lf[(int64_t)min(k0 + j + 5, K) * hw];
+      const float4 d = rows.take(j);
+      bias[0] += d.x; bias[1] += d.y; bias[2] += d.z; bias[3] += d.w;
+#pragma unroll
+      for (int t = 0; t < T; ++t) {
+        acc[t][0] = fmaf(d.x, xs[t], acc[t][0]);
+        acc[t][1] = fmaf(d.y, xs[t], acc[t][1]);
+        acc[t][2] = fmaf(d.z, xs[t], acc[t][2]);
+        acc[t][3] = fmaf(d.w, xs[t], acc[t][3]);
+      }
+    }
+  }
+  quad_grads<T>(acc, bias, g, C, kt, T - kt, gw, gb);
+}
+
+// 3 x 3 stem: grad w[co][tap] += sum dz[k][co] X_nbr(tap)[k]; grad b[co] += sum
+// dz[k][co].  A thread walks kRowsB rows of one column of one step with the X of
+// three rows x three columns in registers: three new X (six log values) and one
+// 16-byte row piece per pixel.  68 bytes per pixel-step (8 clips x 64 x 128 x
+// 128: 1.25 ms with staged pixel-steps, 0.40 without the row ring, now 0.257;
+// HBM floor 0.084).
+constexpr int kRowsB = 32;
+__global__ void __launch_bounds__(256, 2)
+tstem3_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K, int H,
+                  int W, int C, float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ float4 ring[kAhead * 256];
+  const int g = threadIdx.x & 3, pl = (threadIdx.x & 31) >> 2;
+  float acc[9][4] = {}, bias[4] = {};
+  const int64_t hw = (int64_t)H * W;
+  const uint32_t groups = (uint32_t)(W + 7) / 8, strips = (uint32_t)(H + kRowsB - 1) / kRowsB;
+  const uint32_t items = (uint32_t)B * K * strips * groups;
+  for (uint32_t it = blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += gridDim.x * 8) {
+    const int x = (int)(it % groups) * 8 + pl, y0 = (int)(it / groups % strips) * kRowsB;
+    const uint32_t bk = it / groups / strips;
+    if (x >= W) continue;
+    const float* l1 = logl + ((int64_t)(bk / K) * (K + 1) + bk % K + 1) * hw + x;
+    const Rows3 R{l1, l1 - hw, H, W, x > 0, x + 1 < W};
+    const int n = min(kRowsB, H - y0);
+    QuadRing rows{ring + threadIdx.x, dz, bk * hw + (int64_t)y0 * W + x, W, g, C, n};
+    rows.start();
+    float r0[3], r1[3], r2[3], r3[3];
+    R.load(y0 - 1, r0);
+    R.load(y0, r1);
+    R.load(y0 + 1, r2);
+    R.load(y0 + 2, r3);
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      float nx[3];
+      R.load(y0 + j + 3, nx);
+      const float4 d = rows.take(j);
+      bias[0] += d.x; bias[1] += d.y; bias[2] += d.z; bias[3] += d.w;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const float v = t < 3 ? r0[t % 3] : t < 6 ? r1[t % 3] : r2[t % 3];
+        acc[t][0] = fmaf(d.x, v, acc[t][0]);
+        acc[t][1] = fmaf(d.y, v, acc[t][1]);
+        acc[t][2] = fmaf(d.z, v, acc[t][2]);
+        acc[t][3] = fmaf(d.w, v, acc[t][3]);
+      }
+#pragma unroll
+      for (int t = 0; t < 3; ++t) { r0[t] = r1[t]; r1[t] = r2[t]; r2[t] = r3[t]; r3[t] = nx[t]; }
+    }
+  }
+  quad_grads<9>(acc, bias, g, C, 9, 0, gw, gb);
+}
+
 // -------------------------------------- weight backward, spatial stem
-// grad w[co][tap] += sum dz[k][co] X_nbr(tap)[k]; grad b[co] += sum dz[k][co]:
-// the layer-0 kernel above with the taps running over the ks0 x ks0
-// neighbourhood of the current step instead of over time.
+// The other stem sizes (1, 5, 7): persistent blocks stage 128 pixel-steps at a
+// time in shared memory; each thread owns (co, tap) entries, one atomic per
+// entry per block.
+constexpr int kPts = 128;
 __global__ void __launch_bounds__(256)
 tstem_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K, int H,
                  int W, int C, int ks0, float* __restrict__ gw, float* __restrict__ gb) {
@@ -639,18 +882,25 @@ void tlayout(const et_evsnet_weights* net, const et_train_shape* sh, char* base,
 int tforward(const float* logl, const et_train_shape* sh, const et_evsnet_weights* net,
              const TWorkspace& ws, cudaStream_t st) {
   const int C = net->C, L = net->n_layers, kt = net->kt;
-  const int64_t hw = (int64_t)sh->H * sh->W, n = (int64_t)sh->B * sh->K * hw;
-  const unsigned grid = (unsigned)((n + 255) / 256);
+  const int64_t hw = (int64_t)sh->H * sh->W;
   const unsigned grid2 = (unsigned)(((int64_t)sh->B * ((sh->K + 1) / 2) * hw + 255) / 256);   // step pairs
   const int n0 = layer0_taps(net);
   const float* wp = net->w + twofs(L, C, kt, n0);
   const float* bp = net->b + (int64_t)L * C;
-  if (net->ks0 > 0)
-    tstem_fwd<<<grid, 256, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, net->ks0, net->w, net->b,
-                                    ws.act[0], wp, bp, L == 1 ? ws.I : nullptr);
-  else
-    tconv_fwd<<<grid, 256, 0, st>>>(logl, sh->B, sh->K, hw, C, kt, net->w, net->b, ws.act[0], wp, bp,
-                                    L == 1 ? ws.I : nullptr);
+  float* I0 = L == 1 ? ws.I : nullptr;
+  if (net->ks0 == 3) {
+    const int64_t items = (int64_t)sh->B * sh->K * ((sh->H + kRows - 1) / kRows) * ((sh->W + 31) / 32);
+    tstem3_fwd<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, net->w, net->b,
+                                                           ws.act[0], wp, bp, I0);
+  } else if (net->ks0 > 0) {
+    const dim3 grid((unsigned)((hw + 127) / 128), (unsigned)std::min<int64_t>((int64_t)sh->B * sh->K, 65535));
+    tstem_fwd<<<grid, 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, net->ks0, net->w, net->b, ws.act[0], wp,
+                                    bp, I0);
+  } else {
+    const int64_t items = (int64_t)sh->B * ((sh->K + kWalk - 1) / kWalk) * ((hw + 31) / 32);
+    (kt <= 7 ? tconv_fwd<7> : tconv_fwd<9>)<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(
+        logl, sh->B, sh->K, hw, C, kt, net->w, net->b, ws.act[0], wp, bp, I0);
+  }
   ET_CHECK_LAUNCH();
   for (int l = 1; l < L; ++l) {
     // residual form: even layers close a block and add its input
@@ -724,7 +974,7 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
   const unsigned wgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nsm * 8, (n + kPts - 1) / kPts));
   float* dz = ws.g[0];
   const int n0 = layer0_taps(net);
-  tproj_bwd<<<nsm * 4, 256, 0, st>>>(ws.dI, ws.act[L - 1], n, C, net->w + twofs(L, C, kt, n0), dz,
+  tproj_bwd<<<nsm * 8, 256, 0, st>>>(ws.dI, ws.act[L - 1], n, C, net->w + twofs(L, C, kt, n0), dz,
                                      grad_w + twofs(L, C, kt, n0), grad_b + (int64_t)L * C);
   ET_CHECK_LAUNCH();
   const int wthr = twgrad_threads(kt);
@@ -736,10 +986,13 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
       1, std::min<int64_t>((int64_t)nsm * std::max(wblocks, 1), (n + kPts16 - 1) / kPts16));
   auto dkern = C == CP ? tconv16_bwd_data<true> : tconv16_bwd_data<false>;
   auto wgrad = [&](const float* d, int l) -> int {
-    if (l == 0 && net->ks0 > 0)
+    if (l == 0 && net->ks0 == 3)
+      tstem3_bwd_weight<<<nsm * 4, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, grad_w, grad_b);
+    else if (l == 0 && net->ks0 > 0)
       tstem_bwd_weight<<<wgrid, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, net->ks0, grad_w, grad_b);
     else if (l == 0)
-      tconv_bwd_weight<<<wgrid, 256, 0, st>>>(d, logl, B, K, hw, C, kt, grad_w, grad_b);
+      (kt <= 7 ? tconv_bwd_weight<7> : tconv_bwd_weight<9>)<<<nsm * 4, 256, 0, st>>>(
+          d, logl, B, K, hw, C, kt, grad_w, grad_b);
     else if (net->dtype == ET_BF16)
       return et_train_tct_wgrad(d, ws.act[l - 1], B, K, hw, C, kt, grad_w + twofs(l, C, kt, n0),
                                 grad_b + (int64_t)l * C, st);
