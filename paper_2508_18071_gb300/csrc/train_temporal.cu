@@ -17,6 +17,7 @@
 #include "et_internal.cuh"
 #include "evsnet_common.h"
 #include "train_api.h"
+#include "train_tma.cuh"
 
 #define ET_TRY(expr)                 \
   do {                               \
@@ -599,24 +600,14 @@ tstem_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, i
 }
 
 // ------------------------------------------- C -> C layers, vectorised weights
-// The layers with C input channels in a second form: weights staged as
-// [tau][input][output], zero-padded to 16 x 16 per tap, so that one 16-byte
-// shared load (the same address for the whole warp) feeds four FMAs; a
-// pixel-step's 16 channels are read with 16-byte loads when C = 16.
+// The layers with C < 16 input channels: weights staged as [tau][input][output],
+// zero-padded to 16 x 16 per tap, so that one 16-byte shared load (the same
+// address for the whole warp) feeds four FMAs.  (C = 16: the kernels below.)
 constexpr int CP = 16;
 
-template <bool kC16>
 __device__ __forceinline__ void load_ch(const float* __restrict__ src, int C, float (&x)[CP]) {
-  if (kC16) {
 #pragma unroll
-    for (int j = 0; j < CP / 4; ++j) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(src) + j);
-      x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < CP; ++c) x[c] = c < C ? __ldg(src + c) : 0.0f;
-  }
+  for (int c = 0; c < CP; ++c) x[c] = c < C ? __ldg(src + c) : 0.0f;
 }
 
 // acc0[o] += sum_i w[i][o] x0[i] and acc1[o] += sum_i w[i][o] x1[i] for one tap's
@@ -644,14 +635,13 @@ __device__ __forceinline__ void fma_block2(const float* __restrict__ w, const fl
 }
 
 // a pixel-step's channels, zero outside the clip's steps [0, K)
-template <bool kC16>
 __device__ __forceinline__ void load_step(const float* __restrict__ base, int k, int K, int64_t step,
                                           int C, float (&x)[CP]) {
   if (k < 0 || k >= K) {
 #pragma unroll
     for (int c = 0; c < CP; ++c) x[c] = 0.0f;
   } else {
-    load_ch<kC16>(base + k * step, C, x);
+    load_ch(base + k * step, C, x);
   }
 }
 
@@ -659,7 +649,6 @@ __device__ __forceinline__ void load_step(const float* __restrict__ base, int k,
 // also I = bp + wp . out.  One thread per (clip, pair of steps 2j and 2j + 1,
 // pixel): each tap's weights serve both steps, the input of step k - kt + 2 + tau
 // serving the second step at tap tau and the first at tau + 1.
-template <bool kC16>
 __global__ void __launch_bounds__(256, 3)
 tconv16_fwd(const float* __restrict__ in, int B, int K, int64_t hw, int C, int kt,
             const float* __restrict__ w, const float* __restrict__ b, const float* __restrict__ res,
@@ -682,10 +671,10 @@ tconv16_fwd(const float* __restrict__ in, int B, int K, int64_t hw, int C, int k
 #pragma unroll
   for (int co = 0; co < CP; ++co) acc0[co] = acc1[co] = co < C ? b[co] : 0.0f;
   float xa[CP];
-  load_step<kC16>(base, k - (kt - 1), K, step, C, xa);
+  load_step(base, k - (kt - 1), K, step, C, xa);
   for (int tau = 0; tau < kt; ++tau) {
     float xb[CP];
-    load_step<kC16>(base, k - (kt - 1) + tau + 1, K, step, C, xb);
+    load_step(base, k - (kt - 1) + tau + 1, K, step, C, xb);
     fma_block2(sw + tau * CP * CP, xa, xb, C, acc0, acc1);
 #pragma unroll
     for (int c = 0; c < CP; ++c) xa[c] = xb[c];
@@ -700,16 +689,9 @@ tconv16_fwd(const float* __restrict__ in, int B, int K, int64_t hw, int C, int k
       acc[co] = fmaxf(z, 0.0f);
       if (I) Iv += wp[co] * acc[co];
     }
-    if (kC16) {
 #pragma unroll
-      for (int j = 0; j < CP / 4; ++j)
-        reinterpret_cast<float4*>(out + idx * C)[j] =
-            make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-    } else {
-#pragma unroll
-      for (int co = 0; co < CP; ++co)
-        if (co < C) out[idx * C + co] = acc[co];
-    }
+    for (int co = 0; co < CP; ++co)
+      if (co < C) out[idx * C + co] = acc[co];
     if (I) I[idx] = Iv;
   };
   finish(acc0, 0);
@@ -718,7 +700,6 @@ tconv16_fwd(const float* __restrict__ in, int B, int K, int64_t hw, int C, int k
 
 // data backward: out[s][ci] = (add[s][ci] + sum_tau,co w[co][ci][tau] dz[s + kt - 1 - tau][co])
 // 1(mask[s][ci] > 0); weights staged [tau][co][ci]; two steps per thread as above
-template <bool kC16>
 __global__ void __launch_bounds__(256, 3)
 tconv16_bwd_data(const float* __restrict__ dz, int B, int K, int64_t hw, int C, int kt,
                  const float* __restrict__ w, const float* __restrict__ add,
@@ -740,10 +721,10 @@ tconv16_bwd_data(const float* __restrict__ dz, int B, int K, int64_t hw, int C, 
 #pragma unroll
   for (int ci = 0; ci < CP; ++ci) acc0[ci] = acc1[ci] = 0.0f;
   float gb[CP];   // dz[s + kt - tau] for the second step
-  load_step<kC16>(base, s + kt, K, step, C, gb);
+  load_step(base, s + kt, K, step, C, gb);
   for (int tau = 0; tau < kt; ++tau) {
     float ga[CP];
-    load_step<kC16>(base, s + kt - 1 - tau, K, step, C, ga);
+    load_step(base, s + kt - 1 - tau, K, step, C, ga);
     fma_block2(sw + tau * CP * CP, ga, gb, C, acc0, acc1);
 #pragma unroll
     for (int c = 0; c < CP; ++c) gb[c] = ga[c];
@@ -770,7 +751,6 @@ tconv16_bwd_data(const float* __restrict__ dz, int B, int K, int64_t hw, int C, 
 constexpr int kPts16 = 64;
 inline int twgrad_threads(int kt) { return (16 * kt + 16 + 31) / 32 * 32; }
 
-template <bool kC16>
 __global__ void __launch_bounds__(320)
 tconv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, int B, int K,
                    int64_t hw, int C, int kt, float* __restrict__ gw, float* __restrict__ gb) {
@@ -799,31 +779,14 @@ tconv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, i
       }
     }
     __syncthreads();
-    if (kC16) {
-      for (int i = threadIdx.x; i < kPts16 * 4; i += blockDim.x) {
-        const int pt = i >> 2, j = i & 3;
-        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (s_k[pt] >= 0) v = __ldg(reinterpret_cast<const float4*>(dz + (c0 + pt) * CP) + j);
-        reinterpret_cast<float4*>(sd)[i] = v;
-      }
-      for (int i = threadIdx.x; i < kPts16 * kt * 4; i += blockDim.x) {
-        const int pt = i / (kt * 4), r = i % (kt * 4), tt = r >> 2, j = r & 3;
-        const int kk = s_k[pt] - (kt - 1) + tt;
-        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (s_k[pt] >= 0 && kk >= 0)
-          v = __ldg(reinterpret_cast<const float4*>(in + s_row0[pt] + kk * step) + j);
-        reinterpret_cast<float4*>(sx)[i] = v;
-      }
-    } else {
-      for (int i = threadIdx.x; i < kPts16 * CP; i += blockDim.x) {
-        const int pt = i / CP, co = i % CP;
-        sd[i] = (s_k[pt] >= 0 && co < C) ? dz[(c0 + pt) * C + co] : 0.0f;
-      }
-      for (int i = threadIdx.x; i < kPts16 * kt * CP; i += blockDim.x) {
-        const int pt = i / (kt * CP), r = i % (kt * CP), tt = r / CP, ci = r % CP;
-        const int kk = s_k[pt] - (kt - 1) + tt;
-        sx[i] = (s_k[pt] >= 0 && kk >= 0 && ci < C) ? in[s_row0[pt] + kk * step + ci] : 0.0f;
-      }
+    for (int i = threadIdx.x; i < kPts16 * CP; i += blockDim.x) {
+      const int pt = i / CP, co = i % CP;
+      sd[i] = (s_k[pt] >= 0 && co < C) ? dz[(c0 + pt) * C + co] : 0.0f;
+    }
+    for (int i = threadIdx.x; i < kPts16 * kt * CP; i += blockDim.x) {
+      const int pt = i / (kt * CP), r = i % (kt * CP), tt = r / CP, ci = r % CP;
+      const int kk = s_k[pt] - (kt - 1) + tt;
+      sx[i] = (s_k[pt] >= 0 && kk >= 0 && ci < C) ? in[s_row0[pt] + kk * step + ci] : 0.0f;
     }
     __syncthreads();
     if (e < 16 * kt) {
@@ -853,6 +816,351 @@ tconv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, i
   } else if (e < 16 * kt + C) {
     atomicAdd(gb + (e - 16 * kt), bsum);
   }
+}
+
+// ------------------------------------------------- C -> C layers of 16 channels
+// Two FP32 multiply-adds per instruction (each rounded like fmaf): the kernels
+// below are bound by issue slots, of which this takes half; the FP32 pipes give
+// 71 TFLOP/s with either on this device (75 with the pairs).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2f(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2f(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Forward (out = ReLU(b + conv(in) [+ extra]), the last layer also I = bp + wp .
+// out) and data gradient (out = ([extra +] conv^T(in)) 1(mask > 0); in reversed
+// time the same causal convolution) of a layer: each output sums its taps oldest
+// first and, within a tap, channels in order, like tconv16_fwd / _bwd_data.
+// A CTA owns 128 pixels and walks chunks of 8 steps, numbered with time innermost
+// and split evenly over one CTA per SM.  Steps arrive as TMA boxes (64-byte rows,
+// read by each pixel's thread without bank conflicts) in three groups of 8: the
+// previous chunk's (its last kt - 1 steps are this chunk's past), this one's and
+// the next one's.  A thread computes 4 steps of a pixel: a tap's 16 x 16 weights
+// serve 64 pair multiply-adds per 4 weight loads (the same address for the whole
+// warp), 720 instructions per 1024 cycles of the FP32 pipe.
+constexpr int kStepChunk = 8;
+constexpr int kRing = 3 * kStepChunk;
+constexpr uint32_t kTmaPolls = 1u << 24;   // bound of the waits for a box
+
+struct F32ConvArgs {
+  int K, kt;
+  int64_t hw;
+  int tiles, nch;
+  int64_t total;           // B * tiles * nch chunks
+  const float* w;
+  const float* b;
+  const float* extra;
+  const float* mask;
+  float* out;
+  const float* wp;
+  const float* bp;
+  float* I;
+};
+
+template <bool kBwd>
+__global__ void __launch_bounds__(256, 1)
+tconv16_tma(const __grid_constant__ CUtensorMap m_in, F32ConvArgs A) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ uint64_t bar[3];
+  const int tid = threadIdx.x, px = tid & (kBoxPix - 1), half = tid >> 7;
+  const int K = A.K, kt = A.kt, nch = A.nch;
+  float* sw = reinterpret_cast<float*>(sm + kRing * kBox);     // [tau][input][output]
+  for (int i = tid; i < kt * 256; i += 256) {
+    const int tau = i % kt, r = i / kt, lo = r % 16, hi = r / 16;   // w[hi = co][lo = ci][tau]
+    sw[(tau * 16 + (kBwd ? hi : lo)) * 16 + (kBwd ? lo : hi)] = A.w[i];
+  }
+  if (tid == 0)
+    for (int i = 0; i < 3; ++i) mbar_init(&bar[i], 1);
+  __syncthreads();
+  const int64_t t0 = A.total * blockIdx.x / gridDim.x, t1 = A.total * (blockIdx.x + 1) / gridDim.x;
+  // processing order u = 0 .. K-1 is time s = u (forward) or s = K-1-u (data gradient)
+  auto step_of = [&](int u) { return kBwd ? K - 1 - u : u; };
+  // chunk t lives in group (t - t0 + 1) mod 3; thread 0 requests its boxes
+  auto load_chunk = [&](int64_t t) {
+    const int64_t sg = t / nch;
+    const int c = (int)(t - sg * nch), tile = (int)(sg % A.tiles), bc = (int)(sg / A.tiles);
+    const int g = (int)((t - t0 + 1) % 3), n = min(kStepChunk, K - kStepChunk * c);
+    mbar_arrive_expect_tx(&bar[g], (uint32_t)(n * kBox));
+    for (int j = 0; j < n; ++j)
+      tma_load_3d(sm + (g * kStepChunk + j) * kBox, &m_in, 0, tile * kBoxPix, bc * K + step_of(kStepChunk * c + j),
+                  &bar[g]);
+  };
+  const bool mid = t0 % nch != 0;        // the range starts inside a clip: its past is the chunk before
+  if (tid == 0) {
+    if (mid) load_chunk(t0 - 1);
+    if (t0 < t1) load_chunk(t0);
+    if (t0 + 1 < t1) load_chunk(t0 + 1);
+  }
+  uint32_t phase = 0;
+  bool ok = true;
+  if (mid) { ok = mbar_wait(&bar[0], 0, kTmaPolls); phase ^= 1u; }
+  int64_t seg = t0 / nch;
+  int c = (int)(t0 - seg * nch), tile = (int)(seg % A.tiles), bc = (int)(seg / A.tiles);
+  int g = 1;
+  for (int64_t t = t0; t < t1; ++t) {
+    const int gp = g == 0 ? 2 : g - 1;   // the previous chunk's group
+    if (c == 0) {                        // steps before the clip are zero
+      uint4* z = reinterpret_cast<uint4*>(sm + (gp * kStepChunk + kStepChunk - (kt - 1)) * kBox);
+      for (int i = tid; i < (kt - 1) * kBox / 16; i += 256) z[i] = make_uint4(0, 0, 0, 0);
+      __syncthreads();
+    }
+    ok &= mbar_wait(&bar[g], (phase >> g) & 1u, kTmaPolls);
+    phase ^= 1u << g;
+    const int u0 = kStepChunk * c + 4 * half;
+    const int64_t p = (int64_t)tile * kBoxPix + px;
+    if (u0 < K) {
+      f32x2 acc[4][8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const f32x2 b0 = kBwd ? 0ull : pack2f(__ldg(A.b + 2 * i), __ldg(A.b + 2 * i + 1));
+#pragma unroll
+        for (int s = 0; s < 4; ++s) acc[s][i] = b0;
+      }
+      int pos = g * kStepChunk + 4 * half - (kt - 1);   // ring position of the first step's oldest tap
+      if (pos < 0) pos += kRing;
+#pragma unroll 1
+      for (int tau = 0; tau < kt; ++tau) {
+        const unsigned char* row[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) row[s] = sm + (pos + s >= kRing ? pos + s - kRing : pos + s) * kBox;
+        const float* wt = sw + tau * 256;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float4 x[4];
+#pragma unroll
+          for (int s = 0; s < 4; ++s) x[s] = *box_row(row[s], px, q);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            ulonglong2 wv[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) wv[j] = reinterpret_cast<const ulonglong2*>(wt + (4 * q + e) * 16)[j];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+              const float xe = e == 0 ? x[s].x : e == 1 ? x[s].y : e == 2 ? x[s].z : x[s].w;
+              const f32x2 xx = pack2f(xe, xe);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                acc[s][2 * j] = fma2(wv[j].x, xx, acc[s][2 * j]);
+                acc[s][2 * j + 1] = fma2(wv[j].y, xx, acc[s][2 * j + 1]);
+              }
+            }
+          }
+        }
+        pos = pos + 1 == kRing ? 0 : pos + 1;
+      }
+      if (p < A.hw) {
+        float4 ex[4][4], mk[4][4];
+        int64_t idx[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          idx[s] = ((int64_t)bc * K + step_of(min(u0 + s, K - 1))) * A.hw + p;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (A.extra) ex[s][j] = __ldg(reinterpret_cast<const float4*>(A.extra + idx[s] * 16) + j);
+            if (kBwd) mk[s][j] = __ldg(reinterpret_cast<const float4*>(A.mask + idx[s] * 16) + j);
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          if (u0 + s >= K) break;
+          float Iv = (!kBwd && A.I) ? A.bp[0] : 0.0f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float v[4];
+            unpack2f(acc[s][2 * j], v[0], v[1]);
+            unpack2f(acc[s][2 * j + 1], v[2], v[3]);
+            const float e4[4] = {ex[s][j].x, ex[s][j].y, ex[s][j].z, ex[s][j].w};
+            const float m4[4] = {mk[s][j].x, mk[s][j].y, mk[s][j].z, mk[s][j].w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              if (A.extra) v[i] = v[i] + e4[i];
+              if (kBwd) {
+                v[i] = m4[i] > 0.0f ? v[i] : 0.0f;
+              } else {
+                v[i] = fmaxf(v[i], 0.0f);
+                if (A.I) Iv = fmaf(__ldg(A.wp + 4 * j + i), v[i], Iv);
+              }
+              if (!ok) v[i] = __int_as_float(0x7fc00000);   // a box never came
+            }
+            reinterpret_cast<float4*>(A.out + idx[s] * 16)[j] = make_float4(v[0], v[1], v[2], v[3]);
+          }
+          if (!kBwd && A.I) A.I[idx[s]] = ok ? Iv : __int_as_float(0x7fc00000);
+        }
+      }
+    }
+    fence_proxy_async_smem();
+    __syncthreads();
+    // the previous chunk's group is free for the chunk after the next
+    if (tid == 0 && t + 2 < t1) load_chunk(t + 2);
+    g = g == 2 ? 0 : g + 1;
+    if (++c == nch) {
+      c = 0;
+      if (++tile == A.tiles) { tile = 0; ++bc; }
+    }
+  }
+}
+
+// Weight gradient: grad w[co][ci][tau] += sum dz[k][co] in[k - kt + 1 + tau][ci],
+// grad b[co] += sum dz[k][co].  A warp walks two neighbouring pixels through
+// time, lane = (pixel, 4 output channels, 4 input channels): the last T >= kt
+// input rows stay in registers, so a step's two 16-byte reads serve T x 16
+// multiply-adds (T = 7: 56 pair instructions of 66 issued).  The rows come
+// through a ring of kWDepth steps per warp, filled by cp.async (128 bytes of
+// either tensor per step).
+constexpr int kWDepth = 16;
+constexpr int kWWarps = 8;
+template <int T>
+__global__ void __launch_bounds__(32 * kWWarps, 1)
+tconv16_wgrad_walk(const float* __restrict__ dz, const float* __restrict__ in, int B, int K, int64_t hw, int kt,
+                   int seg, float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ __align__(16) float ring[kWWarps][kWDepth][2][2][16];   // [step][dz, in][pixel][channel]
+  __shared__ float sum[T * 256 + 16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pix = lane >> 4, cq = lane & 3, iq = (lane >> 2) & 3;
+  f32x2 acc[T][4][2];
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+#pragma unroll
+    for (int a = 0; a < 4; ++a) acc[t][a][0] = acc[t][a][1] = 0ull;
+  float bias[4] = {};
+  const uint32_t pairs = (uint32_t)((hw + 1) / 2), segs = (uint32_t)(K + seg - 1) / seg;
+  const uint32_t items = (uint32_t)B * segs * pairs;   // rows that fit the device: below 2^32
+  for (uint32_t it = blockIdx.x * kWWarps + warp; it < items; it += gridDim.x * kWWarps) {
+    const int64_t p0 = (int64_t)(it % pairs) * 2;
+    const int k0 = (int)(it / pairs % segs) * seg, bc = (int)(it / pairs / segs);
+    const int k1 = min(K, k0 + seg), kb = max(0, k0 - (kt - 1));   // steps kb .. k0 - 1 only fill the registers
+    const bool live = p0 + pix < hw;
+    // lanes 0-15 copy 16 bytes each of a step's rows
+    const int lt = (lane >> 3) & 1, lp = (lane >> 2) & 1, lc = lane & 3;
+    const bool copy = lane < 16 && p0 + lp < hw;
+    const float* src = (lt ? in : dz) + (((int64_t)bc * K) * hw + p0 + lp) * 16 + 4 * lc;
+    auto request = [&](int k) {
+      if (copy && k < k1)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         smem_u32(&ring[warp][k & (kWDepth - 1)][lt][lp][4 * lc])),
+                     "l"(src + (int64_t)k * hw * 16)
+                     : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    __syncwarp();                        // the ring of the previous item has been read
+#pragma unroll
+    for (int j = 0; j < kWDepth - 1; ++j) request(kb + j);
+    f32x2 xr[T][2];                      // input rows of the last T steps, row of step kb + j at j mod T
+#pragma unroll
+    for (int t = 0; t < T; ++t) xr[t][0] = xr[t][1] = 0ull;
+    for (int kk = kb; kk < k1; kk += T) {
+#pragma unroll
+      for (int r = 0; r < T; ++r) {
+        const int k = kk + r;
+        if (k < k1) {
+          asm volatile("cp.async.wait_group %0;" ::"n"(kWDepth - 2) : "memory");
+          __syncwarp();                  // every lane's copies of step k have landed; step k - 1 has been read
+          request(k + kWDepth - 1);
+          const float(*row)[2][16] = ring[warp][k & (kWDepth - 1)];
+          float4 d = *reinterpret_cast<const float4*>(&row[0][pix][4 * cq]);
+          ulonglong2 x = *reinterpret_cast<const ulonglong2*>(&row[1][pix][4 * iq]);
+          if (!live) x.x = x.y = 0ull;
+          if (!live || k < k0) d = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          xr[r][0] = x.x;
+          xr[r][1] = x.y;
+          const float dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+          for (int a = 0; a < 4; ++a) {
+            bias[a] += dv[a];
+            const f32x2 dd = pack2f(dv[a], dv[a]);
+#pragma unroll
+            for (int t = 0; t < T; ++t) {   // tap t of T meets the row of step k - (T - 1) + t
+              const f32x2(&xt)[2] = xr[(r + 1 + t) % T];
+              acc[t][a][0] = fma2(dd, xt[0], acc[t][a][0]);
+              acc[t][a][1] = fma2(dd, xt[1], acc[t][a][1]);
+            }
+          }
+        }
+      }
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  for (int i = threadIdx.x; i < T * 256 + 16; i += blockDim.x) sum[i] = 0.0f;
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float lo, hi;
+        unpack2f(acc[t][a][h], lo, hi);
+        lo += __shfl_xor_sync(0xFFFFFFFFu, lo, 16);
+        hi += __shfl_xor_sync(0xFFFFFFFFu, hi, 16);
+        if (lane < 16) {
+          float* e = &sum[(t * 16 + 4 * cq + a) * 16 + 4 * iq + 2 * h];
+          atomicAdd(e, lo);
+          atomicAdd(e + 1, hi);
+        }
+      }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    float v = bias[a] + __shfl_xor_sync(0xFFFFFFFFu, bias[a], 16);
+    if (lane < 4) atomicAdd(&sum[T * 256 + 4 * cq + a], v);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kt * 256; i += blockDim.x) {   // gw[co][ci][tau]
+    const int tau = i % kt, ci = i / kt % 16, co = i / (kt * 16);
+    atomicAdd(gw + i, sum[((tau + T - kt) * 16 + co) * 16 + ci]);
+  }
+  if (threadIdx.x < 16) atomicAdd(gb + threadIdx.x, sum[T * 256 + threadIdx.x]);
+}
+
+int sm_count(int* n) {
+  int dev = 0;
+  ET_CHECK_CUDA(cudaGetDevice(&dev));
+  ET_CHECK_CUDA(cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev));
+  return ET_OK;
+}
+
+int launch_conv_tma(bool data_grad, const float* in, int B, int K, int64_t hw, int kt, const float* w,
+                    const float* b, const float* extra, const float* mask, float* out, const float* wp,
+                    const float* bp, float* I, cudaStream_t st) {
+  const int64_t tiles = (hw + kBoxPix - 1) / kBoxPix, nch = (K + kStepChunk - 1) / kStepChunk;
+  F32ConvArgs A{K, kt, hw, (int)tiles, (int)nch, B * tiles * nch, w, b, extra, mask, out, wp, bp, I};
+  CUtensorMap m_in;
+  ET_TRY(map_rows(&m_in, in, (int64_t)B * K, hw));
+  int nsm = 0;
+  ET_TRY(sm_count(&nsm));
+  const int smem = kRing * kBox + kt * 256 * (int)sizeof(float);
+  auto kern = data_grad ? tconv16_tma<true> : tconv16_tma<false>;
+  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  kern<<<(unsigned)std::min<int64_t>(A.total, nsm), 256, smem, st>>>(m_in, A);
+  ET_CHECK_LAUNCH();
+  return ET_OK;
+}
+
+int launch_wgrad_walk(const float* dz, const float* in, int B, int K, int64_t hw, int kt, float* gw, float* gb,
+                      cudaStream_t st) {
+  int nsm = 0;
+  ET_TRY(sm_count(&nsm));
+  // whole clips per warp, or segments of at least 16 steps (each rereads the
+  // kt - 1 steps before it) when there are fewer than two pixel pairs per warp
+  const int64_t pairs = (hw + 1) / 2 * B, want = 2ll * nsm * kWWarps;
+  int seg = K;
+  if (pairs < want) seg = (int)std::max<int64_t>(16, K / std::max<int64_t>(1, want / pairs));
+  auto kern = kt <= 3 ? tconv16_wgrad_walk<3> : kt <= 5 ? tconv16_wgrad_walk<5>
+              : kt <= 7 ? tconv16_wgrad_walk<7> : tconv16_wgrad_walk<9>;
+  const int64_t items = pairs * ((K + seg - 1) / seg);
+  kern<<<(unsigned)std::min<int64_t>((items + kWWarps - 1) / kWWarps, nsm), 32 * kWWarps, 0, st>>>(
+      dz, in, B, K, hw, kt, seg, gw, gb);
+  ET_CHECK_LAUNCH();
+  return ET_OK;
 }
 
 struct TWorkspace {
@@ -912,8 +1220,13 @@ int tforward(const float* logl, const et_train_shape* sh, const et_evsnet_weight
       if (rc != ET_OK) return rc;
       continue;
     }
-    auto kern = C == CP ? tconv16_fwd<true> : tconv16_fwd<false>;
-    kern<<<grid2, 256, 0, st>>>(ws.act[l - 1], sh->B, sh->K, hw, C, kt, net->w + twofs(l, C, kt, n0),
+    if (use_tma(sh->B, sh->K, hw, C, ws.act[l - 1], ws.act[l])) {
+      ET_TRY(launch_conv_tma(false, ws.act[l - 1], sh->B, sh->K, hw, kt, net->w + twofs(l, C, kt, n0),
+                             net->b + (int64_t)l * C, res, nullptr, ws.act[l], wp, bp, l == L - 1 ? ws.I : nullptr,
+                             st));
+      continue;
+    }
+    tconv16_fwd<<<grid2, 256, 0, st>>>(ws.act[l - 1], sh->B, sh->K, hw, C, kt, net->w + twofs(l, C, kt, n0),
                                net->b + (int64_t)l * C, res, ws.act[l], wp, bp,
                                l == L - 1 ? ws.I : nullptr);
     ET_CHECK_LAUNCH();
@@ -979,12 +1292,10 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
   ET_CHECK_LAUNCH();
   const int wthr = twgrad_threads(kt);
   const size_t wsmem = sizeof(float) * kPts16 * CP * (1 + kt);
-  auto wkern = C == CP ? tconv16_bwd_weight<true> : tconv16_bwd_weight<false>;
   int wblocks = 0;   // resident weight-gradient blocks per SM: one wave of persistent blocks
-  ET_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wblocks, wkern, wthr, wsmem));
+  ET_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wblocks, tconv16_bwd_weight, wthr, wsmem));
   const unsigned wgrid16 = (unsigned)std::max<int64_t>(
       1, std::min<int64_t>((int64_t)nsm * std::max(wblocks, 1), (n + kPts16 - 1) / kPts16));
-  auto dkern = C == CP ? tconv16_bwd_data<true> : tconv16_bwd_data<false>;
   auto wgrad = [&](const float* d, int l) -> int {
     if (l == 0 && net->ks0 == 3)
       tstem3_bwd_weight<<<nsm * 4, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, grad_w, grad_b);
@@ -996,8 +1307,11 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
     else if (net->dtype == ET_BF16)
       return et_train_tct_wgrad(d, ws.act[l - 1], B, K, hw, C, kt, grad_w + twofs(l, C, kt, n0),
                                 grad_b + (int64_t)l * C, st);
+    else if (use_tma(B, K, hw, C, d, ws.act[l - 1]))
+      return launch_wgrad_walk(d, ws.act[l - 1], B, K, hw, kt, grad_w + twofs(l, C, kt, n0),
+                               grad_b + (int64_t)l * C, st);
     else
-      wkern<<<wgrid16, wthr, wsmem, st>>>(d, ws.act[l - 1], B, K, hw, C, kt, grad_w + twofs(l, C, kt, n0),
+      tconv16_bwd_weight<<<wgrid16, wthr, wsmem, st>>>(d, ws.act[l - 1], B, K, hw, C, kt, grad_w + twofs(l, C, kt, n0),
                                           grad_b + (int64_t)l * C);
     return ET_OK;
   };
@@ -1006,7 +1320,10 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
     if (net->dtype == ET_BF16)
       return et_train_tct_conv(d, B, K, hw, C, kt, net->w + twofs(l, C, kt, n0), nullptr, add, mask, out,
                                nullptr, nullptr, nullptr, true, st);
-    dkern<<<grid2, 256, 0, st>>>(d, B, K, hw, C, kt, net->w + twofs(l, C, kt, n0), add, mask, out);
+    if (use_tma(B, K, hw, C, d, out))
+      return launch_conv_tma(true, d, B, K, hw, kt, net->w + twofs(l, C, kt, n0), nullptr, add, mask, out, nullptr,
+                             nullptr, nullptr, st);
+    tconv16_bwd_data<<<grid2, 256, 0, st>>>(d, B, K, hw, C, kt, net->w + twofs(l, C, kt, n0), add, mask, out);
     return ET_OK;
   };
   if (net->kind == ET_NET_STACK) {
