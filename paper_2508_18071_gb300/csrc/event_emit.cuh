@@ -30,3 +30,78 @@ __device__ __forceinline__ void emit_events_warp(et_event* events, int64_t cap,
     out[3 * slot + 2] = (uint32_t)(uint8_t)(int8_t)p;
   }
 }
+
+// A warp's events gathered in shared memory and appended kCap at a time: the
+// appends of all warps meet on one counter, whose atomics the device serves one
+// after the other (a 25-frame 720p call with an append per warp and step makes
+// 720,000 of them), and an append's round trip holds its warp up.  An event is
+// packed as (step - base) << 6 | lane << 1 | (p > 0); x and y are the lane's.
+template <int kCap>
+struct EventStage {
+  uint32_t* buf;        // the warp's kCap entries in shared memory
+  int n = 0;            // entries held (the same in every lane)
+  uint32_t base = 0;    // step of the packed entries' zero
+  et_event* events;
+  int64_t cap;
+  unsigned long long* counter;
+  uint32_t x, y, t0;    // the lane's pixel; label of step 0
+
+  __device__ __forceinline__ EventStage(uint32_t* buf_, et_event* events_, int64_t cap_,
+                                        unsigned long long* counter_, uint32_t x_, uint32_t y_, uint32_t t0_)
+      : buf(buf_), events(events_), cap(cap_), counter(counter_), x(x_), y(y_), t0(t0_) {}
+
+  __device__ __forceinline__ void flush() {
+    if (n == 0) return;
+    const unsigned lane = threadIdx.x & 31u;
+    __syncwarp();
+    unsigned long long at = 0;
+    if (lane == 0) at = atomicAdd(counter, (unsigned long long)n);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    uint32_t* out = reinterpret_cast<uint32_t*>(events);
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + (int)lane;
+      const uint32_t e = i < n ? buf[i] : 0u;
+      const uint32_t xy = __shfl_sync(0xFFFFFFFFu, x | (y << 16), (e >> 1) & 31u);
+      const unsigned long long slot = at + (unsigned long long)i;
+      if (i < n && slot < (unsigned long long)cap) {
+        out[3 * slot] = xy;
+        out[3 * slot + 1] = t0 + base + (e >> 6);
+        out[3 * slot + 2] = (e & 1u) ? 1u : 0xFFu;
+      }
+    }
+    __syncwarp();
+    n = 0;
+  }
+
+  // every lane of the warp calls this: cnt events of polarity p at `step`
+  // (steps never fall below the smallest step of an earlier call by more than
+  // the caller's window, `first` = the smallest step any lane passes)
+  __device__ __forceinline__ void add(uint32_t cnt, uint32_t step, uint32_t first, int p) {
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned any = __ballot_sync(0xFFFFFFFFu, cnt != 0);
+    if (!any) return;
+    int rank = __popc(any & ((1u << lane) - 1u)), total = __popc(any);
+    if (__any_sync(0xFFFFFFFFu, cnt > 1)) {
+      // more than the entries hold from one lane alone: counted in full, and
+      // the append below then goes straight to the buffer
+      const uint32_t c = min(cnt, (uint32_t)kCap + 1u);
+      uint32_t incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (unsigned)o) incl += v;
+      }
+      rank = (int)(incl - c);
+      total = (int)__shfl_sync(0xFFFFFFFFu, incl, 31);
+      if (total > kCap) {
+        emit_events_warp(events, cap, counter, cnt, x, y, t0 + step, p);
+        return;
+      }
+    }
+    if (n + total > kCap || first + (1u << 20) - base >= (1u << 25)) flush();
+    if (n == 0) base = first;
+    for (uint32_t i = 0; i < cnt; ++i)
+      buf[n + rank + (int)i] = ((step - base) << 6) | (lane << 1) | (p > 0 ? 1u : 0u);
+    n += total;
+  }
+};
