@@ -18,6 +18,7 @@
 #include "evsnet_common.h"
 #include "train_api.h"
 #include "train_tma.cuh"
+#include "f32x2.cuh"
 
 #define ET_TRY(expr)                 \
   do {                               \
@@ -819,24 +820,6 @@ tconv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, i
 }
 
 // ------------------------------------------------- C -> C layers of 16 channels
-// Two FP32 multiply-adds per instruction (each rounded like fmaf): the kernels
-// below are bound by issue slots, of which this takes half; the FP32 pipes give
-// 71 TFLOP/s with either on this device (75 with the pairs).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2f(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2f(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // Forward (out = ReLU(b + conv(in) [+ extra]), the last layer also I = bp + wp .
 // out) and data gradient (out = ([extra +] conv^T(in)) 1(mask > 0); in reversed
 // time the same causal convolution) of a layer: each output sums its taps oldest
