@@ -35,7 +35,8 @@ __device__ __forceinline__ void emit_events_warp(et_event* events, int64_t cap,
 // appends of all warps meet on one counter, whose atomics the device serves one
 // after the other (a 25-frame 720p call with an append per warp and step makes
 // 720,000 of them), and an append's round trip holds its warp up.  An event is
-// packed as (step - base) << 6 | lane << 1 | (p > 0); x and y are the lane's.
+// packed as (step - base) << 11 | dy << 6 | lane << 1 | (p > 0); x and y are the
+// lane's, y plus dy rows (dy < 32).
 template <int kCap>
 struct EventStage {
   uint32_t* buf;        // the warp's kCap entries in shared memory
@@ -64,8 +65,8 @@ struct EventStage {
       const uint32_t xy = __shfl_sync(0xFFFFFFFFu, x | (y << 16), (e >> 1) & 31u);
       const unsigned long long slot = at + (unsigned long long)i;
       if (i < n && slot < (unsigned long long)cap) {
-        out[3 * slot] = xy;
-        out[3 * slot + 1] = t0 + base + (e >> 6);
+        out[3 * slot] = xy + (((e >> 6) & 31u) << 16);
+        out[3 * slot + 1] = t0 + base + (e >> 11);
         out[3 * slot + 2] = (e & 1u) ? 1u : 0xFFu;
       }
     }
@@ -73,10 +74,10 @@ struct EventStage {
     n = 0;
   }
 
-  // every lane of the warp calls this: cnt events of polarity p at `step`
-  // (steps never fall below the smallest step of an earlier call by more than
-  // the caller's window, `first` = the smallest step any lane passes)
-  __device__ __forceinline__ void add(uint32_t cnt, uint32_t step, uint32_t first, int p) {
+  // every lane of the warp calls this: cnt events of polarity p at `step`, dy
+  // rows below the lane's pixel (`first` = the smallest step any lane passes, at
+  // most 2^15 below it; it never decreases from call to call)
+  __device__ __forceinline__ void add(uint32_t cnt, uint32_t step, uint32_t first, int p, uint32_t dy = 0) {
     const unsigned lane = threadIdx.x & 31u;
     const unsigned any = __ballot_sync(0xFFFFFFFFu, cnt != 0);
     if (!any) return;
@@ -94,14 +95,41 @@ struct EventStage {
       rank = (int)(incl - c);
       total = (int)__shfl_sync(0xFFFFFFFFu, incl, 31);
       if (total > kCap) {
-        emit_events_warp(events, cap, counter, cnt, x, y, t0 + step, p);
+        emit_events_warp(events, cap, counter, cnt, x, y + dy, t0 + step, p);
         return;
       }
     }
-    if (n + total > kCap || first + (1u << 20) - base >= (1u << 25)) flush();
+    if (n + total > kCap || first + (1u << 15) - base >= (1u << 20)) flush();
     if (n == 0) base = first;
     for (uint32_t i = 0; i < cnt; ++i)
-      buf[n + rank + (int)i] = ((step - base) << 6) | (lane << 1) | (p > 0 ? 1u : 0u);
+      buf[n + rank + (int)i] = ((step - base) << 11) | (dy << 6) | (lane << 1) | (p > 0 ? 1u : 0u);
     n += total;
+  }
+
+  // every lane of the warp calls this: bit k of `fired` is an event at `step`,
+  // dy0 + k rows below the lane's pixel, negative where bit k of `neg` is set
+  // (32 kRows <= kCap)
+  template <int kRows>
+  __device__ __forceinline__ void add_rows(uint32_t fired, uint32_t neg, uint32_t step, uint32_t dy0) {
+    static_assert(32 * kRows <= kCap, "a call's events fit the entries");
+    const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+    if (!__any_sync(0xFFFFFFFFu, fired != 0)) return;
+    unsigned m[kRows];
+    int total = 0;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+      m[k] = __ballot_sync(0xFFFFFFFFu, (fired >> k) & 1u);
+      total += __popc(m[k]);
+    }
+    if (n + total > kCap || step + (1u << 15) - base >= (1u << 20)) flush();
+    if (n == 0) base = step;
+    const uint32_t e = ((step - base) << 11) | (dy0 << 6) | (lane << 1);
+    int at = n;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+      if ((fired >> k) & 1u) buf[at + __popc(m[k] & below)] = e + ((uint32_t)k << 6) + (((neg >> k) & 1u) ^ 1u);
+      at += __popc(m[k]);
+    }
+    n = at;
   }
 };

@@ -11,6 +11,10 @@ int et_evsnet_forward_f32(const float* logl, int32_t F, const et_evsnet_weights*
 int et_evsnet_forward_tc(const float* logl, int32_t F, const et_evsnet_weights* net,
                          et_evsnet_state* st, int32_t t0, et_event* events, int64_t cap,
                          int64_t* n_events, float* I_out, int8_t* spikes, cudaStream_t stream);
+// its BF16 form for at most 16 channels (2 to 6 layers of 3x3, checked there)
+int et_evsnet_forward_tc16(const float* logl, int32_t F, const et_evsnet_weights* net,
+                           et_evsnet_state* st, int32_t t0, et_event* events, int64_t cap,
+                           int64_t* n_events, float* I_out, int8_t* spikes, cudaStream_t stream);
 int et_evsnet_forward_pix(const float* logl, int32_t F, const et_evsnet_weights* net,
                           et_evsnet_state* st, int32_t t0, et_event* events, int64_t cap,
                           int64_t* n_events, float* I_out, int8_t* spikes, cudaStream_t stream);

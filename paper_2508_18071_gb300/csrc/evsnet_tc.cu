@@ -1,6 +1,7 @@
 // EvSNet forward on the tcgen05 tensor cores for the spatial form: a stack of
 // 3x3 convolutions with ReLU (Eq. 5 with kernel extent in space), the
-// point-wise projection (Eq. 6) and BiLIF (Eq. 2-3), for up to 32 channels.
+// point-wise projection (Eq. 6) and BiLIF (Eq. 2-3), for up to 32 channels
+// (BF16 with at most 16: evsnet_tc16.cu, which takes three taps per MMA).
 // Two operand precisions, FP32 accumulation in TMEM for both:
 //   BF16 (kind::f16): weights and layer inputs rounded to BF16;
 //   FP8  (kind::f8f6f4, E4M3): weights scaled per output channel and layer
@@ -469,7 +470,7 @@ int et_evsnet_forward_tc(const float* logl, int32_t F, const et_evsnet_weights* 
   const bool f8 = net->dtype == ET_FP8;
   if (net->C <= 16)
     return f8 ? launch<16, true>(logl, F, net, st, t0, events, cap, n_events, I_out, spikes, stream)
-              : launch<16, false>(logl, F, net, st, t0, events, cap, n_events, I_out, spikes, stream);
+              : et_evsnet_forward_tc16(logl, F, net, st, t0, events, cap, n_events, I_out, spikes, stream);
   return f8 ? launch<32, true>(logl, F, net, st, t0, events, cap, n_events, I_out, spikes, stream)
             : launch<32, false>(logl, F, net, st, t0, events, cap, n_events, I_out, spikes, stream);
 }
