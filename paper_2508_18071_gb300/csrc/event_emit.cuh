@@ -107,9 +107,9 @@ struct EventStage {
   }
 
   // every lane of the warp calls this: bit k of `fired` is an event at `step`,
-  // dy0 + k rows below the lane's pixel, negative where bit k of `neg` is set
-  // (32 kRows <= kCap)
-  template <int kRows>
+  // dy0 + k rows below the lane's pixel (or, kSteps, at step + k and dy0 rows
+  // below), negative where bit k of `neg` is set (32 kRows <= kCap)
+  template <int kRows, bool kSteps = false>
   __device__ __forceinline__ void add_rows(uint32_t fired, uint32_t neg, uint32_t step, uint32_t dy0) {
     static_assert(32 * kRows <= kCap, "a call's events fit the entries");
     const unsigned lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
@@ -127,7 +127,8 @@ struct EventStage {
     int at = n;
 #pragma unroll
     for (int k = 0; k < kRows; ++k) {
-      if ((fired >> k) & 1u) buf[at + __popc(m[k] & below)] = e + ((uint32_t)k << 6) + (((neg >> k) & 1u) ^ 1u);
+      if ((fired >> k) & 1u) buf[at + __popc(m[k] & below)] =
+            e + ((uint32_t)k << (kSteps ? 11 : 6)) + (((neg >> k) & 1u) ^ 1u);
       at += __popc(m[k]);
     }
     n = at;

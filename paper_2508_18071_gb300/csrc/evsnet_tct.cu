@@ -5,7 +5,8 @@
 // (the weights of layers 1.. and their inputs), FP32 accumulation in TMEM;
 // layer 0, the residual sums, the projection and BiLIF stay FP32.
 //
-// A CTA owns a tile of 128 consecutive pixels for the whole call: one TMEM
+// One CTA per SM (shared memory, TMEM) walks tiles of 128 consecutive pixels,
+// each for the whole call, with the weights staged once: one TMEM
 // lane per pixel and three groups of 128 threads, one thread per pixel each
 // (warps w, w + 4, w + 8 share TMEM lane quarter w); group g runs the
 // epilogues of every third tensor-core layer counting down from the last, so
@@ -64,16 +65,33 @@
 // orders in both precisions: results depend on a step's place in its pair
 // (FP32 rounding), so calls with even step counts reproduce one call exactly.
 //
+// What bounds it: the chain of a round (layer 0's and the epilogues' CUDA-core
+// work between two barriers, ~7 k clk for two steps of 128 pixels against ~1.5 k
+// of MMAs), and per tile reading and writing the FP32 history (20 k and 11 k clk;
+// at 1280x720 3.1 GB a call).  Hence the kernel is compiled per form (no
+// runtime choice of stem or input path inside the round), layer 0 and the
+// epilogues run on FP32 pairs (fma.rn.f32x2, bit-identical to fmaf) with 16-byte
+// weight loads, events are gathered per warp, and the history moves a channel row
+// of 128 pixels at a time in 16-byte pieces (32-bit ones where a row is not
+// 16-byte aligned).  Measured, 1280x720, paper form behind the 3 x 3 stem: 128 ->
+// 94 us per step and 1692 -> 1206 per call in BF16, 127 -> 86 and 2002 -> 1260 in
+// FP8; 253x187: 9.9 -> 7.2 and 117 -> 103, 10.1 -> 8.2 and 136 -> 112; no stem,
+// 1280x720: 157 -> 147 and 1738 -> 1425.  One CTA per tile with the same rounds had
+// 1601 and 1909 per call; prefetching the next tile's history into L2 and cached
+// instead of streaming history accesses changed nothing.
+//
 // MMA waits are bounded; on expiry the kernel sets bit 62 of the event count,
 // leaves the membrane and history state untouched, waits (bounded) for its
 // MMAs in flight and frees its TMEM.
 #include "et_internal.cuh"
 #include "event_emit.cuh"
 #include "evsnet_common.h"
+#include "f32x2.cuh"
 #include "tc_ptx.cuh"
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
+#include <algorithm>
 #include <cstring>
 
 namespace {
@@ -101,6 +119,7 @@ constexpr int kHbCol = (kMaxLayers - 1) * kT * 16;
 constexpr uint32_t kTmemCols = 512;
 static_assert(kHbCol + 3 * 3 * kT * 16 <= (int)kTmemCols, "TMEM columns");
 constexpr unsigned long long kTimeoutBit = 1ull << 62;
+constexpr int kStageCap = 64;           // events a warp of group 0 holds before it appends them
 constexpr uint32_t kDrainIters = 1u << 22;   // bound of the waits for work in flight after a bail
 
 struct TctParams {
@@ -111,6 +130,7 @@ struct TctParams {
   int woff[kMaxLayers + 1];             // packed weight offsets per layer (+ projection)
   int off_wB, off_f32, off_xbuf;        // shared-memory byte offsets
   int tma;                              // the stem's input tiles come by TMA
+  int tiles;                            // tiles of TP pixels
   uint32_t wait_iters;
   const float* scales;                  // FP8: input scale of tensor-core layer l at [l - 1]
   unsigned int* amax;                   // calibration: largest input of layer l + 1 at [l] (float bits), or NULL
@@ -218,7 +238,11 @@ __device__ __forceinline__ void load_row8(const unsigned char* slot, int m, floa
   }
 }
 
-template <bool kF8, bool kCal>
+// kForm, the layer 0 a kernel is compiled for (one kernel for all of them is 150 KB
+// of code, more than the instruction cache, of which a round touches pieces in all
+// three worker groups): 0 temporal, 3 the 3 x 3 stem by thread loads, 4 the 3 x 3
+// stem by TMA, -1 any (calibration, other stem sizes)
+template <bool kF8, bool kCal, int kForm>
 __global__ void __launch_bounds__(kThreads, 1)
 evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const float* __restrict__ logl,
                   const float* __restrict__ wg, const float* __restrict__ bg, float* __restrict__ Vg,
@@ -230,8 +254,9 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   __shared__ uint64_t tma_bar[2];       // the two TMA box buffers
   __shared__ uint64_t drain_bar;
   __shared__ uint32_t tmem_slot;
-  __shared__ int bail;
-  const int L = P.L, C = P.C, kt = P.kt, R = P.R, hk = kt - 1, ks0 = P.ks0;
+  __shared__ uint32_t staged[TP / 32][kStageCap];   // group 0's events
+  const int L = P.L, C = P.C, kt = P.kt, R = P.R, hk = kt - 1, ks0 = kForm < 0 ? P.ks0 : kForm == 4 ? 3 : kForm;
+  constexpr bool kTma = kForm == 4;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int p = tid & (TP - 1);         // pixel of the tile = TMEM lane
   const int grp = tid >> 7;             // worker group (4 = the issuing warp)
@@ -240,7 +265,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   // group 0), so that consecutive layers' epilogues run in different warps
   auto owns = [&](int l) { return (L - 1 - l) % kGroups == grp; };
   const int64_t npix = (int64_t)P.H * P.W;
-  const int64_t q = (int64_t)blockIdx.x * TP + p;
+  int64_t q = 0;                        // this thread's pixel of the current tile
   const bool worker = tid < kWorkers;
   const bool stem_grp = grp == kStemGroup;
   // layer 0: the stem group alone (BF16), or split by channel halves between
@@ -250,8 +275,8 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   constexpr int kSC = kF8 ? CP / 2 : CP;          // layer-0 channels per participating thread
   const bool stem_part = kF8 ? (grp == 1 || grp == 2) : stem_grp;
   const int c_lo = (kF8 && grp == 2) ? CP / 2 : 0;   // its first channel
-  const bool live = worker && q < npix;
-  const int px = live ? (int)(q % P.W) : 0, py = live ? (int)(q / P.W) : 0;
+  bool live = false, failed = false;    // failed: a bounded wait of this thread gave up
+  int px = 0, py = 0;
   constexpr int kSB = kF8 ? kSlot8 : kSlot;                    // bytes per ring slot
   // slots per layer.  FP8: positions R .. RS - 1 repeat 0 .. RS - R - 1; a
   // window starts below R and its slot pairs end at kt + 1 (kt odd) or kt + 2
@@ -359,34 +384,12 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
       reinterpret_cast<uint4*>(rings)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
   }
-  // ring slots of steps -(kt-1) .. -1 from the state (oldest first): group g
-  // fills the slots j with j % 3 == g (both channel halves), a layer's loads
-  // issued before its stores
-  for (int l = 1; l < L; ++l) {
-    constexpr int kJ = (kMaxKt - 1 + kGroups - 1) / kGroups;
-    float v[kJ][CP];
-#pragma unroll
-    for (int jj = 0; jj < kJ; ++jj) {
-      const int j = jj * kGroups + grp;
-#pragma unroll
-      for (int c = 0; c < CP; ++c) v[jj][c] = (j < hk && live && c < C) ? hist[hidx(l, j, c)] : 0.0f;
-    }
-#pragma unroll
-    for (int jj = 0; jj < kJ; ++jj) {
-      const int j = jj * kGroups + grp;
-      if (worker && j < hk) put_row(l, ring_pos(j - hk, R), v[jj]);
-    }
-  }
-  if (ks0 == 0 && stem_grp)
-    for (int j = 0; j < hk; ++j) xh[ring_pos(j - hk, R) * TP + p] = live ? hist[hidx(0, j, 0)] : 0.0f;
-  float V = (live && grp == 0) ? Vg[q] : 0.0f;
   if (warp == 0) tmem_alloc(&tmem_slot, kTmemCols);
   if (tid == 0) {
     for (int l = 0; l < kMaxLayers; ++l) mbar_init(&lbar[l], 1);
     mbar_init(&tma_bar[0], 1);
     mbar_init(&tma_bar[1], 1);
     mbar_init(&drain_bar, 1);
-    bail = 0;
   }
   tc_fence_before();
   __syncthreads();
@@ -411,9 +414,9 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
 
   const int S = P.F - P.f0;             // steps of this call
   const int nch = (S + kT - 1) / kT;    // chunks of kT steps
-  // 3 x 3 stem: the nine neighbours' X of the steps of a chunk, loaded a chunk
-  // ahead so that their latency hides behind the tensor-core layers
-  float xn[kT][9];
+  // 3 x 3 stem without TMA: the nine neighbours' X of the steps of a chunk, loaded
+  // a chunk ahead so that their latency hides behind the tensor-core layers
+  float xa[kT][9];
   auto load_x9 = [&](int s_first) {
 #pragma unroll
     for (int j = 0; j < kT; ++j) {
@@ -425,14 +428,13 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
         const int64_t qq = in ? (int64_t)yy * P.W + xx : 0;
         const float xc = in ? __ldg(logl + (int64_t)f * npix + qq) : 0.0f;
         const float xp = !in ? 0.0f : (f == 0 ? last_l[qq] : __ldg(logl + (int64_t)(f - 1) * npix + qq));
-        xn[j][t] = xc - xp;
+        xa[j][t] = xc - xp;
       }
     }
   };
-  if (ks0 == 3 && stem_part) load_x9(0);
   // TMA of the stem's input: the tile's row segment (tiles are whole row
   // segments when it is used), one box per chunk, two buffers
-  const int tx0 = (int)(((int64_t)blockIdx.x * TP) % P.W), ty0 = (int)(((int64_t)blockIdx.x * TP) / P.W);
+  int tx0 = 0, ty0 = 0;
   uint32_t tma_phase[2] = {0u, 0u};     // stem group: parity of the next completion per buffer
   int tma_issued[2] = {0, 0};           // issuing thread: boxes issued per buffer
   auto issue_box = [&](int ch) {
@@ -449,71 +451,110 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   auto stem = [&](int ch) {
     float h0n[kT][kSC];
     const int s0 = ch * kT, tc = min(kT, S - s0);
-    if (P.tma && ch > 0) {
+    float xn[kT][9];
+    if (kTma) {
       const int b = ch & 1;
-      if (!mbar_wait(&tma_bar[b], tma_phase[b], P.wait_iters)) {
-        if (lane == 0) atomicOr(n_events, kTimeoutBit);
-        bail = 1;
+      if (ch > 0) {                      // chunk 0's box was filled by the threads
+        if (!mbar_wait(&tma_bar[b], tma_phase[b], P.wait_iters)) {
+          if (lane == 0) atomicOr(n_events, kTimeoutBit);
+          failed = true;
+        }
+        tma_phase[b] ^= 1u;
       }
-      tma_phase[b] ^= 1u;
-      const float* xb = xbuf + b * kBoxStride;
+      const float* xb = xbuf + b * kBoxStride + p + 3;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        float l[kT + 1];
+#pragma unroll
+        for (int j = 0; j <= kT; ++j) l[j] = xb[(j * 3 + t / 3) * kBoxW + t % 3];
+#pragma unroll
+        for (int j = 0; j < kT; ++j) xn[j][t] = l[j + 1] - l[j];
+      }
+    } else if (ks0 == 3) {
+#pragma unroll
+      for (int t = 0; t < 9; ++t)
+#pragma unroll
+        for (int j = 0; j < kT; ++j) xn[j][t] = xa[j][t];
+    }
+    f32x2 acc[kT][kSC / 2];
+#pragma unroll
+    for (int c = 0; c < kSC / 4; ++c) {
+      const ulonglong2 b2 = *reinterpret_cast<const ulonglong2*>(bs + c_lo + 4 * c);
+#pragma unroll
+      for (int j = 0; j < kT; ++j) { acc[j][2 * c] = b2.x; acc[j][2 * c + 1] = b2.y; }
+    }
+    // a tap's weights for the steps it meets (a pixel past the end: its values are never used)
+    auto tap = [&](int t, const float (&x)[kT]) {
+      f32x2 d[kT];
+#pragma unroll
+      for (int j = 0; j < kT; ++j) d[j] = pack2f(x[j], x[j]);
+#pragma unroll
+      for (int c = 0; c < kSC / 4; ++c) {
+        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(w0 + t * CP + c_lo + 4 * c);
+#pragma unroll
+        for (int j = 0; j < kT; ++j) {
+          acc[j][2 * c] = fma2(w.x, d[j], acc[j][2 * c]);
+          acc[j][2 * c + 1] = fma2(w.y, d[j], acc[j][2 * c + 1]);
+        }
+      }
+    };
+    if (ks0 == 3) {
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        float x[kT];
+#pragma unroll
+        for (int j = 0; j < kT; ++j) x[j] = xn[j][t];
+        tap(t, x);
+      }
+    } else if (ks0 > 0) {
+      const int r0 = ks0 >> 1;
+      for (int dy = 0; dy < ks0; ++dy) {
+        const int yy = py + dy - r0;
+        if (yy < 0 || yy >= P.H) continue;
+        for (int dx = 0; dx < ks0; ++dx) {
+          const int xx = px + dx - r0;
+          if (xx < 0 || xx >= P.W) continue;
+          const int64_t qq = (int64_t)yy * P.W + xx;
+          float x[kT];
+#pragma unroll
+          for (int j = 0; j < kT; ++j) {
+            const int f = P.f0 + s0 + j;
+            x[j] = 0.0f;
+            if (j < tc)
+              x[j] = __ldg(logl + (int64_t)f * npix + qq) -
+                     (f == 0 ? last_l[qq] : __ldg(logl + (int64_t)(f - 1) * npix + qq));
+          }
+          tap(dy * ks0 + dx, x);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < kT; ++j) {
+        if (j >= tc || !live) continue;
+        const int f = P.f0 + s0 + j;
+        xh[ring_pos(s0 + j, R) * TP + p] = __ldg(logl + (int64_t)f * npix + q) -
+                                           (f == 0 ? last_l[q] : __ldg(logl + (int64_t)(f - 1) * npix + q));
+      }
+      for (int t = 0; t < kt; ++t) {
+        float x[kT];
+#pragma unroll
+        for (int j = 0; j < kT; ++j) x[j] = j < tc ? xh[ring_pos(s0 + j - hk + t, R) * TP + p] : 0.0f;
+        tap(t, x);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kT; ++j)
+#pragma unroll
+      for (int c = 0; c < kSC / 2; ++c) {
+        unpack2f(acc[j][c], h0n[j][2 * c], h0n[j][2 * c + 1]);
+        h0n[j][2 * c] = fmaxf(h0n[j][2 * c], 0.0f);
+        h0n[j][2 * c + 1] = fmaxf(h0n[j][2 * c + 1], 0.0f);
+      }
+    if (kCal)
 #pragma unroll
       for (int j = 0; j < kT; ++j)
 #pragma unroll
-        for (int t = 0; t < 9; ++t) {
-          const int col = p + t % 3 + 3, row = t / 3;
-          xn[j][t] = xb[((1 + j) * 3 + row) * kBoxW + col] - xb[(j * 3 + row) * kBoxW + col];
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < kT; ++j) {
-#pragma unroll
-      for (int c = 0; c < kSC; ++c) h0n[j][c] = 0.0f;
-      if (j >= tc) continue;
-      const int f = P.f0 + s0 + j;
-      float acc[kSC];
-#pragma unroll
-      for (int c = 0; c < kSC; ++c) acc[c] = bs[c_lo + c];
-      if (live) {
-        if (ks0 == 3) {
-#pragma unroll
-          for (int t = 0; t < 9; ++t) {
-            const float* wt = w0 + t * CP + c_lo;
-#pragma unroll
-            for (int c = 0; c < kSC; ++c) acc[c] = fmaf(wt[c], xn[j][t], acc[c]);
-          }
-        } else if (ks0 > 0) {
-          const int r0 = ks0 >> 1;
-          for (int dy = 0; dy < ks0; ++dy) {
-            const int yy = py + dy - r0;
-            if (yy < 0 || yy >= P.H) continue;
-            for (int dx = 0; dx < ks0; ++dx) {
-              const int xx = px + dx - r0;
-              if (xx < 0 || xx >= P.W) continue;
-              const int64_t qq = (int64_t)yy * P.W + xx;
-              const float xc = __ldg(logl + (int64_t)f * npix + qq);
-              const float xp = f == 0 ? last_l[qq] : __ldg(logl + (int64_t)(f - 1) * npix + qq);
-              const float v = xc - xp;
-              const float* wt = w0 + (dy * ks0 + dx) * CP + c_lo;
-#pragma unroll
-              for (int c = 0; c < kSC; ++c) acc[c] = fmaf(wt[c], v, acc[c]);
-            }
-          }
-        } else {
-          const float xc = __ldg(logl + (int64_t)f * npix + q);
-          const float xp = f == 0 ? last_l[q] : __ldg(logl + (int64_t)(f - 1) * npix + q);
-          xh[ring_pos(s0 + j, R) * TP + p] = xc - xp;
-          for (int tau0 = 0; tau0 < kt; ++tau0) {
-            const float v = xh[ring_pos(s0 + j - hk + tau0, R) * TP + p];
-            const float* wt = w0 + tau0 * CP + c_lo;
-#pragma unroll
-            for (int c = 0; c < kSC; ++c) acc[c] = fmaf(wt[c], v, acc[c]);
-          }
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kSC; ++c) h0n[j][c] = live ? fmaxf(acc[c], 0.0f) : 0.0f;
-    }
+        for (int c = 0; c < kSC; ++c) h0n[j][c] = live && j < tc ? h0n[j][c] : 0.0f;
     if (residual && L >= 3) {
       // the first block's FP32 input: columns (step j, channel c) = 16 j + c
       if constexpr (kSC == CP) tmem_st32(hb_col(0, ch), &h0n[0][0]);
@@ -562,14 +603,74 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
       }
     }
   };
-  // chunk 0 before the first round (its previous frame may be the state's:
-  // thread loads), chunk 1's box in flight
-  if (tid == kIssuer && P.tma && nch > 1) issue_box(1);
-  if (stem_part && nch > 0) {
-    stem(0);
-    stem_store(0);
-    if (ks0 == 3 && !P.tma) load_x9(kT);
+  EventStage<kStageCap> stage(staged[warp & 3], events, cap, n_events, 0u, 0u, (uint32_t)P.t0);
+  bool bail = false;
+  // the history's pieces: kHistCh channels of one ring slot
+  constexpr int kHistCh = kF8 ? CP : kHalf, kPlanes = CP / kHistCh;
+  const int hist_items = (L - 1) * hk * kPlanes;
+  // four pixels per lane and access where the rows allow it
+  const bool vec = npix % 4 == 0 && (reinterpret_cast<uintptr_t>(hist) & 15) == 0;
+  for (int tile = blockIdx.x; tile < P.tiles; tile += gridDim.x) {
+  q = (int64_t)tile * TP + p;
+  live = worker && q < npix;
+  px = live ? (int)(q % P.W) : 0;
+  py = live ? (int)(q / P.W) : 0;
+  tx0 = (int)(((int64_t)tile * TP) % P.W);
+  ty0 = (int)(((int64_t)tile * TP) / P.W);
+  stage.x = (uint32_t)px;
+  stage.y = (uint32_t)py;
+  const int np = (int)min((int64_t)TP, npix - (int64_t)tile * TP);   // pixels of the tile
+  float V = (live && grp == 0) ? Vg[q] : 0.0f;
+  // ring slots of steps -(kt-1) .. -1 from the state (oldest first).  A channel's
+  // 128 pixels are 512 bytes, the next channel's lie npix on -- in another page:
+  // a warp takes eight (FP8: sixteen) channels of a slot whole, four consecutive
+  // loads per channel, so that a page is looked up once (a thread per pixel going
+  // through the channels looked up every page four times, and the lookups, not the
+  // bytes, took 20 k to 50 k clocks per tile)
+  if (worker) {
+#pragma unroll 1
+    for (int it = warp; it < hist_items; it += kWorkers / 32) {
+      const int pl = it % kPlanes, j = it / kPlanes % hk, l = 1 + it / (kPlanes * hk);
+      const float* h = hist + (((int64_t)l * hk + j) * C + pl * kHistCh) * npix + (int64_t)tile * TP;
+      float v[4][kHistCh];
+#pragma unroll
+      for (int c = 0; c < kHistCh; ++c) {
+        const bool on = pl * kHistCh + c < C;
+        if (vec) {
+          const float4 r = on && 4 * lane < np ? __ldcs(reinterpret_cast<const float4*>(h + c * npix) + lane)
+                                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          v[0][c] = r.x; v[1][c] = r.y; v[2][c] = r.z; v[3][c] = r.w;
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[i][c] = on && lane + 32 * i < np ? __ldcs(h + c * npix + lane + 32 * i) : 0.0f;
+        }
+      }
+      const int pos = ring_pos(j - hk, R);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int m = vec ? 4 * lane + i : lane + 32 * i;
+        if constexpr (kF8)
+          store_row8(slot_of(l, pos), pos + R < RS ? slot_of(l, pos + R) : nullptr, m, v[i], isc[l]);
+        else
+          *reinterpret_cast<uint4*>(slot_of(l, pos) + pl * kPlane + m * 16) =
+              make_uint4(pack_bf16(v[i][0], v[i][1]), pack_bf16(v[i][2], v[i][3]), pack_bf16(v[i][4], v[i][5]),
+                         pack_bf16(v[i][6], v[i][7]));
+      }
+    }
   }
+  if (kTma && nch > 0) {
+    // chunk 0's box, whose previous frame may be the state's, by thread loads
+    for (int i = tid; i < kBoxFloats; i += kThreads) {
+      const int x = tx0 - 4 + i % kBoxW, y = ty0 - 1 + i / kBoxW % 3, f = P.f0 - 1 + i / (3 * kBoxW);
+      const bool in = x >= 0 && x < P.W && y >= 0 && y < P.H && f < P.F;
+      const int64_t qq = in ? (int64_t)y * P.W + x : 0;
+      xbuf[i] = !in ? 0.0f : f < 0 ? last_l[qq] : __ldg(logl + (int64_t)f * npix + qq);
+    }
+  } else if (ks0 == 3 && stem_part && nch > 0) {
+    load_x9(0);
+  }
+  if (ks0 == 0 && stem_grp)
+    for (int j = 0; j < hk; ++j) xh[ring_pos(j - hk, R) * TP + p] = live ? hist[hidx(0, j, 0)] : 0.0f;
   // Rounds: in round tau tensor-core layer l computes chunk tau - l + 1 and
   // layer 0 chunk tau + 1, so that one MMA issue and one barrier serve every
   // layer, and layer 0's CUDA-core work runs while the MMAs do.  Layer l's
@@ -577,19 +678,20 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   // that layer l + 1's MMAs of the same round read: the MMAs are issued last
   // layer first and each epilogue waits for its own layer's commit, which
   // follows every later layer's MMAs; layer 0's output is stored after layer
-  // 1's commit, the round's last.
-  for (int tau = 0; tau < nch + L - 2; ++tau) {
+  // 1's commit, the round's last.  Round -1 is layer 0 of chunk 0 alone.
+#pragma unroll 1
+  for (int tau = -1; tau < nch + L - 2; ++tau) {
     // ---- every tensor-core layer's MMAs, last layer first
     fence_proxy_async_smem();
     tc_fence_before();
-    __syncthreads();
+    bail = __syncthreads_or(failed) != 0;
     tc_fence_after();
     if (bail) break;
     if (tid == kIssuer) {
       // the box of chunk tau + 2, into the buffer chunk tau's layer 0 read in
       // the previous round (every thread's proxy fence before the barrier above
       // orders those reads first)
-      if (P.tma && tau + 2 < nch) issue_box(tau + 2);
+      if (kTma && tau + 2 < nch) issue_box(tau + 2);
       constexpr uint64_t kBlock = (CP * 16) >> 4;   // one 16-row block of the strip
       constexpr uint64_t kSlotU = kSlot >> 4;
       // layer l's chunk this round starts at step 2 (tau - l + 1); its first
@@ -641,7 +743,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
     // ---- layer 0 of the next chunk, in registers, while the MMAs run
     if (stem_part && tau + 1 < nch) {
       stem(tau + 1);
-      if (ks0 == 3 && !P.tma) load_x9((tau + 2) * kT);   // consumed next round
+      if (ks0 == 3 && !kTma) load_x9((tau + 2) * kT);   // consumed next round
     }
     // ---- this group's epilogues, last layer first, each after its layer's commit
     for (int l = L - 1; l >= 1 && worker; --l) {
@@ -650,9 +752,9 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
       if (c < 0 || c >= nch) continue;
       const int s0 = c * kT, tc = min(kT, S - s0), pc = ring_pos(s0, R);
       if (!mbar_wait(&lbar[l], (lphase >> l) & 1u, P.wait_iters)) {
-        // give up: the results are not used (the state is left untouched)
+        // give up: the results are not used (the tile's state is left untouched)
         if (lane == 0) atomicOr(n_events, kTimeoutBit);
-        bail = 1;
+        failed = true;
       }
       lphase ^= 1u << l;
       tc_fence_after();
@@ -663,15 +765,37 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
       if (closing) tmem_ld32x2(acc_col(l), hb_col(l / 2 - 1, c), acc, hin);
       else tmem_ld32(acc_col(l), acc);
       float Is[kT];
+      const ulonglong2* b2 = reinterpret_cast<const ulonglong2*>(bs + l * CP);
 #pragma unroll
       for (int j = 0; j < kT; ++j) {
         float* out = acc + j * CP;      // the outputs replace the accumulators
 #pragma unroll
-        for (int c2 = 0; c2 < CP; ++c2) {
-          // FP8: the accumulators carry the weight and input scales
-          const float v = kF8 ? fmaf(out[c2], dq[l * CP + c2], bs[l * CP + c2]) : out[c2] + bs[l * CP + c2];
-          const float o = closing ? fmaxf(hin[j * CP + c2] + v, 0.0f) : fmaxf(v, 0.0f);
-          out[c2] = (live && j < tc) ? o : 0.0f;
+        for (int c4 = 0; c4 < CP / 4; ++c4) {
+          const ulonglong2 b = b2[c4];
+          float* o = out + 4 * c4;
+          f32x2 v0, v1;
+          if constexpr (kF8) {
+            // the accumulators carry the weight and input scales
+            const ulonglong2 d = reinterpret_cast<const ulonglong2*>(dq + l * CP)[c4];
+            v0 = fma2(pack2f(o[0], o[1]), d.x, b.x);
+            v1 = fma2(pack2f(o[2], o[3]), d.y, b.y);
+          } else {
+            v0 = add2(pack2f(o[0], o[1]), b.x);
+            v1 = add2(pack2f(o[2], o[3]), b.y);
+          }
+          if (closing) {
+            const float* h = hin + j * CP + 4 * c4;
+            v0 = add2(pack2f(h[0], h[1]), v0);
+            v1 = add2(pack2f(h[2], h[3]), v1);
+          }
+          unpack2f(v0, o[0], o[1]);
+          unpack2f(v1, o[2], o[3]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            o[e] = fmaxf(o[e], 0.0f);
+            // a pixel past the end and a step past the last are stored nowhere that counts
+            if (kCal) o[e] = live && j < tc ? o[e] : 0.0f;
+          }
         }
         if (l + 1 < L) {
           if (j < tc) put_row(l + 1, pc + j >= R ? pc + j - R : pc + j, out);
@@ -679,7 +803,13 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
           // Eq. 6 projection
           Is[j] = bp[0];
 #pragma unroll
-          for (int c2 = 0; c2 < CP; ++c2) Is[j] = fmaf(wp[c2], out[c2], Is[j]);
+          for (int c4 = 0; c4 < CP / 4; ++c4) {
+            const float4 w = *reinterpret_cast<const float4*>(wp + 4 * c4);
+            Is[j] = fmaf(w.x, out[4 * c4], Is[j]);
+            Is[j] = fmaf(w.y, out[4 * c4 + 1], Is[j]);
+            Is[j] = fmaf(w.z, out[4 * c4 + 2], Is[j]);
+            Is[j] = fmaf(w.w, out[4 * c4 + 3], Is[j]);
+          }
         }
       }
       // a closing layer's output is the next block's input
@@ -694,33 +824,30 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
       }
       if (l == L - 1) {
         // BiLIF (Eq. 2-3) step by step and the events
+        uint32_t fired = 0, neg = 0;
 #pragma unroll
         for (int j = 0; j < kT; ++j) {
-          if (j >= tc) break;
-          const int f = P.f0 + s0 + j;
-          uint32_t nev = 0;
-          int Sp = 0;
-          if (live) {
-            const float I = Is[j];
-            const float vp = P.beta * V + I;
-            Sp = vp >= P.vth ? 1 : (vp <= -P.vth ? -1 : 0);
-            V = vp - P.reset * (float)Sp;
-            nev = (Sp != 0 && P.t0 + f >= 0) ? 1u : 0u;   // delayed labels below 0: none
-            const int64_t o = (int64_t)(s0 + j) * npix + q;
-            if (I_out) I_out[o] = I;
-            if (spikes) spikes[o] = (int8_t)Sp;
-          }
-          emit_events_warp(events, cap, n_events, nev, (uint32_t)px, (uint32_t)py, (uint32_t)(P.t0 + f), Sp);
+          if (j >= tc || !live) break;
+          const float I = Is[j];
+          const float vp = P.beta * V + I;
+          const int Sp = vp >= P.vth ? 1 : (vp <= -P.vth ? -1 : 0);
+          V = vp - P.reset * (float)Sp;
+          if (Sp != 0 && P.t0 + P.f0 + s0 + j >= 0) fired |= 1u << j;   // delayed labels below 0: none
+          if (Sp < 0) neg |= 1u << j;
+          const int64_t o = (int64_t)(s0 + j) * npix + q;
+          if (I_out) I_out[o] = I;
+          if (spikes) spikes[o] = (int8_t)Sp;
         }
+        stage.template add_rows<kT, true>(fired, neg, (uint32_t)(P.f0 + s0), 0u);
       }
     }
     // layer 1's MMAs of this round are complete once its commit has arrived:
     // chunk tau + 1 may then overwrite the ring slots they read
     if (stem_part && tau + 1 < nch) {
-      if (!owns(1)) {
+      if (tau >= 0 && !owns(1)) {
         if (!mbar_wait(&lbar[1], (lphase >> 1) & 1u, P.wait_iters)) {
           if (lane == 0) atomicOr(n_events, kTimeoutBit);
-          bail = 1;
+          failed = true;
         }
         lphase ^= 2u;
       }
@@ -729,7 +856,47 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
     tmem_wait_st();
     tc_fence_before();
   }
-  __syncthreads();
+  bail |= __syncthreads_or(failed) != 0;
+  if (bail) break;
+  // layer 0's group waits for layer 1's commit in every round but the last chunk's
+  if (stem_part && !owns(1) && nch > 0) lphase ^= 2u;
+  if (worker) {
+    if (grp == 0) stage.flush();
+    if (live && grp == 0) Vg[q] = V;
+    // the last kt - 1 inputs of every layer back to the state, oldest first, in the
+    // same pieces
+#pragma unroll 1
+    for (int it = warp; it < hist_items; it += kWorkers / 32) {
+      const int pl = it % kPlanes, j = it / kPlanes % hk, l = 1 + it / (kPlanes * hk);
+      const unsigned char* slot = slot_of(l, ring_pos(S - hk + j, R));
+      float* h = hist + (((int64_t)l * hk + j) * C + pl * kHistCh) * npix + (int64_t)tile * TP;
+      float v[4][kHistCh];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int m = vec ? 4 * lane + i : lane + 32 * i;
+        if constexpr (kF8) load_row8(slot, m, scl[l], v[i]);
+        else load_half(slot, pl, m, v[i]);
+      }
+#pragma unroll
+      for (int c = 0; c < kHistCh; ++c) {
+        if (pl * kHistCh + c >= C) continue;
+        if (vec) {
+          if (4 * lane < np)
+            __stcs(reinterpret_cast<float4*>(h + c * npix) + lane, make_float4(v[0][c], v[1][c], v[2][c], v[3][c]));
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (lane + 32 * i < np) __stcs(h + c * npix + lane + 32 * i, v[i][c]);
+        }
+      }
+    }
+    if (live) {
+      if (ks0 == 0 && stem_grp)
+        for (int j = 0; j < hk; ++j) hist[hidx(0, j, 0)] = xh[ring_pos(S - hk + j, R) * TP + p];
+    }
+  }
+  __syncthreads();                      // the rings have been read
+  }
   if (bail) {
     // a bounded wait gave up: one more commit tracks every MMA still in
     // flight; wait for it, and for the TMA, with a second bounded wait
@@ -738,20 +905,6 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
     if (tid == kIssuer)
       for (int b = 0; b < 2; ++b)
         if (tma_issued[b] > 0) mbar_wait(&tma_bar[b], (uint32_t)((tma_issued[b] - 1) & 1), kDrainIters);
-  } else if (live) {
-    if (grp == 0) Vg[q] = V;
-    // the last kt - 1 inputs of every layer back to the state, oldest first
-    // (group g the slots j with j % 3 == g)
-    for (int l = 1; l < L; ++l)
-      for (int j = grp; j < hk; j += kGroups) {
-        float v[CP];
-        if constexpr (kF8) load_row8(slot_of(l, ring_pos(S - hk + j, R)), p, scl[l], v);
-        else load_row(slot_of(l, ring_pos(S - hk + j, R)), p, v);
-        for (int c = 0; c < CP; ++c)
-          if (c < C) hist[hidx(l, j, c)] = v[c];
-      }
-    if (ks0 == 0 && stem_grp)
-      for (int j = 0; j < hk; ++j) hist[hidx(0, j, 0)] = xh[ring_pos(S - hk + j, R) * TP + p];
   }
   tc_fence_before();
   __syncthreads();
@@ -800,7 +953,7 @@ int tct_launch(const float* logl, int32_t F, const et_evsnet_weights* net, et_ev
   // base and row pitch 16-byte aligned
   CUtensorMap tmap;
   std::memset(&tmap, 0, sizeof(tmap));
-  P.tma = P.ks0 == 3 && P.W % TP == 0 && (reinterpret_cast<uintptr_t>(logl) & 15) == 0 && F >= 1;
+  P.tma = !amax && P.ks0 == 3 && P.W % TP == 0 && (reinterpret_cast<uintptr_t>(logl) & 15) == 0 && F >= 1;
   P.off_xbuf = (int)(((size_t)P.off_f32 + fbytes + 127) & ~(size_t)127);
   const size_t smem = (size_t)P.off_xbuf + (P.tma ? (size_t)(kBoxStride + kBoxFloats) * 4 : 0);
   if (P.tma) {
@@ -828,16 +981,26 @@ int tct_launch(const float* logl, int32_t F, const et_evsnet_weights* net, et_ev
   int dev = 0, max_smem = 0;
   ET_CHECK_CUDA(cudaGetDevice(&dev));
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  int nsm = 0;
+  ET_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   // static shared memory (barriers, TMEM slot, flag) comes on top of the dynamic part
-  auto kern = f8 ? evsnet_tct_kernel<true, false>
-                 : (amax ? evsnet_tct_kernel<false, true> : evsnet_tct_kernel<false, false>);
+  const int form = P.tma ? 4 : (P.ks0 == 0 || P.ks0 == 3) ? P.ks0 : -1;
+  auto kern = evsnet_tct_kernel<false, true, -1>;
+  if (!amax && f8)
+    kern = form == 4 ? evsnet_tct_kernel<true, false, 4> : form == 3 ? evsnet_tct_kernel<true, false, 3>
+           : form == 0 ? evsnet_tct_kernel<true, false, 0> : evsnet_tct_kernel<true, false, -1>;
+  else if (!amax)
+    kern = form == 4 ? evsnet_tct_kernel<false, false, 4> : form == 3 ? evsnet_tct_kernel<false, false, 3>
+           : form == 0 ? evsnet_tct_kernel<false, false, 0> : evsnet_tct_kernel<false, false, -1>;
   cudaFuncAttributes fa;
   ET_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
   if (smem + fa.sharedSizeBytes > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
   if (P.kt > 1 && !st->hist) return ET_ERR_ARG;
   ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int64_t npix = (int64_t)P.H * P.W;
-  kern<<<(unsigned)((npix + TP - 1) / TP), kThreads, smem, stream>>>(
+  P.tiles = (int)(((int64_t)P.H * P.W + TP - 1) / TP);
+  // one CTA per SM (shared memory, TMEM), each walking tiles: the weights are staged
+  // once (a CTA per tile: 400 us more per 1280x720 call)
+  kern<<<(unsigned)std::min(P.tiles, nsm), kThreads, smem, stream>>>(
       tmap, P, logl, net->w, net->b, st->V, st->hist, st->last_l, events, cap,
       reinterpret_cast<unsigned long long*>(n_events), I_out, spikes);
   ET_CHECK_LAUNCH();
