@@ -22,6 +22,7 @@
 #include <cuda.h>
 #include "et_internal.cuh"
 #include "evsnet_common.h"
+#include "f32x2.cuh"
 #include "train_api.h"
 
 namespace {
@@ -253,225 +254,308 @@ conv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, in
 }
 
 // ------------------------------------------- C -> C layers, register-blocked
-// The layers with C input channels (all but the first) in a second form: the
-// 16 x 16 tile (+ halo) of all channels is staged channel-interleaved in shared
-// memory, 16 floats per position, the four 16-byte groups of position m
-// permuted by (m >> 1) & 3 so that eight consecutive positions read a group
-// from eight different bank quads.  Channels are zero-padded to 16.
+// FP32 convolutions with C input channels (all layers but the first), channels
+// zero-padded to 16.  What bounds them is the FP32 pipe once shared memory is read
+// rarely enough: a warp's 16-byte load takes 4 clk of the SM's 128 bytes per clk
+// whatever its addresses, as long as 4 multiply-adds of the SM.
 constexpr int CP = 16;
-constexpr int TP = TS + 2;     // tile with halo
+constexpr int CW = 32;             // columns of a tile: a warp's lanes
+constexpr int kRows = 8;           // rows of one warp's forward tile
+constexpr int kPitch = CW + 2;     // a staged row with its halo
+constexpr int kWTap = CP * CP + 4; // words of a tap's staged weights (4 apart: fewer bank conflicts when staging)
 
-__device__ __forceinline__ int cidx(int m, int g) { return m * CP + 4 * (g ^ ((m >> 1) & 3)); }
-
-// plane-major [c][y][x] tile (rows y0 - h .., columns x0 - h .., tw x th) ->
-// interleaved shared memory; zero outside the image and for c >= C
-__device__ __forceinline__ void stage(float* __restrict__ s, const float* __restrict__ g, int C,
-                                      int H, int W, int x0, int y0, int h, int tw, int th) {
-  const int64_t hw = (int64_t)H * W;
-  for (int i = threadIdx.x; i < CP * tw * th; i += blockDim.x) {
-    const int c = i / (tw * th), r = i % (tw * th);
-    const int yy = y0 - h + r / tw, xx = x0 - h + r % tw;
-    float v = 0.0f;
-    if (c < C && yy >= 0 && yy < H && xx >= 0 && xx < W) v = g[(int64_t)c * hw + (int64_t)yy * W + xx];
-    s[cidx(r, c >> 2) + (c & 3)] = v;
-  }
+// 4 bytes global -> shared without a register; zero when !ok
+__device__ __forceinline__ void copy4(float* dst, const float* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(ok ? 4 : 0));
 }
 
-// acc[k][c] += sum over taps t and input channels of wt[t][ci][4 cg + c] x[m_k + off(t)][ci]
-// (off(t) = (t / 3 - 1, t % 3 - 1) on a TP-wide tile); 4 positions x 4 channels
-// per thread, 8 vector loads per 64 FMAs
-__device__ __forceinline__ void conv_block(const float* __restrict__ sx, const float* __restrict__ wt,
-                                           const int (&m)[4], int cg, float (&acc)[4][4]) {
+// Forward (out = ReLU(b + conv(in)); the last layer also I = bp + wp . out) or, kBwd,
+// the data gradient: dzp[ci] = (sum_co,t w[co][ci][t] dz[co] at the mirrored tap)
+// 1(mask > 0), i.e. the same sum with weights w'[t][co][ci] = w[co][ci][8 - t].
+// A block of two warps owns 8 rows x 32 columns of an image; the input lies in
+// shared memory by channel planes, a lane owns a column: 8 rows x 8 output
+// channels (a half per warp) of sums as FP32 pairs, so that 8 four-byte loads and two
+// 16-byte weight loads feed 64 multiply-adds (16 clk of shared memory for 16 of
+// the FP32 pipe; 4 positions x 4 channels took 32).  Every sum runs over taps, then
+// channels, in one chain of fused multiply-adds.  Up to seven blocks per SM hide each
+// other's staging; 32 images of 93 x 67 are one wave of 864 blocks.  Average launch over
+// a training pass on 50 steps of two such clips (segments of 32 and 4 images): forward
+// 41 -> 25 us, data gradient 42 -> 31.  Single multiply-adds instead of pairs: 27 and 33;
+// four warps on 16 rows (480 blocks, 3.2 per SM): 30 and 41.
+template <bool kBwd>
+__global__ void __launch_bounds__(64, 7)
+conv16(const float* __restrict__ in, int C, int H, int W, const float* __restrict__ w,
+       const float* __restrict__ b, float* __restrict__ out, const float* __restrict__ wp,
+       const float* __restrict__ bp, float* __restrict__ I, const float* __restrict__ mask) {
+  constexpr int kSR = kRows + 2, kPlane = kSR * kPitch;
+  __shared__ __align__(16) float sw[9 * kWTap];     // [t][from][to]
+  __shared__ float sx[CP * kPlane];                 // [channel][row][column]
+  __shared__ uint32_t son[2][kBwd ? 64 : 1];
+  const int n = blockIdx.z, tx = (W + CW - 1) / CW, x0 = blockIdx.x % tx * CW, y0 = blockIdx.x / tx * kRows;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t hw = (int64_t)H * W;
+  const float* img = in + (int64_t)n * C * hw + (int64_t)(y0 - 1) * W + x0 - 1;
+  {
+    const bool okx = x0 - 1 + lane >= 0 && x0 - 1 + lane < W;
 #pragma unroll 1
-  for (int t = 0; t < 9; ++t) {
-    const int toff = (t / 3 - 1) * TP + (t % 3 - 1);
-    const float* w = wt + t * CP * CP + 4 * cg;
-    int mk[4];
+    for (int c = warp * 8; c < warp * 8 + 8; ++c) {
+      const float* src = img + c * hw + lane;
+      float* dst = sx + c * kPlane + lane;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) mk[k] = m[k] + toff;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const float4 wa = *reinterpret_cast<const float4*>(w + (4 * g + 0) * CP);
-      const float4 wb = *reinterpret_cast<const float4*>(w + (4 * g + 1) * CP);
-      const float4 wc = *reinterpret_cast<const float4*>(w + (4 * g + 2) * CP);
-      const float4 wd = *reinterpret_cast<const float4*>(w + (4 * g + 3) * CP);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float4 x = *reinterpret_cast<const float4*>(sx + cidx(mk[k], g));
-        acc[k][0] = fmaf(wa.x, x.x, acc[k][0]); acc[k][1] = fmaf(wa.y, x.x, acc[k][1]);
-        acc[k][2] = fmaf(wa.z, x.x, acc[k][2]); acc[k][3] = fmaf(wa.w, x.x, acc[k][3]);
-        acc[k][0] = fmaf(wb.x, x.y, acc[k][0]); acc[k][1] = fmaf(wb.y, x.y, acc[k][1]);
-        acc[k][2] = fmaf(wb.z, x.y, acc[k][2]); acc[k][3] = fmaf(wb.w, x.y, acc[k][3]);
-        acc[k][0] = fmaf(wc.x, x.z, acc[k][0]); acc[k][1] = fmaf(wc.y, x.z, acc[k][1]);
-        acc[k][2] = fmaf(wc.z, x.z, acc[k][2]); acc[k][3] = fmaf(wc.w, x.z, acc[k][3]);
-        acc[k][0] = fmaf(wd.x, x.w, acc[k][0]); acc[k][1] = fmaf(wd.y, x.w, acc[k][1]);
-        acc[k][2] = fmaf(wd.z, x.w, acc[k][2]); acc[k][3] = fmaf(wd.w, x.w, acc[k][3]);
+      for (int r = 0; r < kSR; ++r) {
+        const bool ok = okx && c < C && (unsigned)(y0 - 1 + r) < (unsigned)H;
+        copy4(dst + r * kPitch, ok ? src + r * W : in, ok);
       }
     }
+    // the two columns right of the lanes', lane = (row, column) of a channel
+    const int r = tid >> 1 & 15, col = CW + (tid & 1);
+    const bool ok = (unsigned)(y0 - 1 + r) < (unsigned)H && x0 - 1 + col < W;
+    if (r < kSR)
+#pragma unroll 4
+      for (int c = tid >> 5; c < CP; c += 2)
+        copy4(sx + c * kPlane + r * kPitch + col, ok && c < C ? img + c * hw + r * W + col : in, ok && c < C);
   }
-}
-
-// Thread layout of the 256-thread blocks below: warp w, lane (pg = lane / 4,
-// cg = lane % 4) computes channels 4 cg .. 4 cg + 3 at the tile positions
-// w * 32 + k * 8 + pg, k = 0..3.
-__device__ __forceinline__ void tile_positions(int (&pix)[4], int (&m)[4]) {
-  const int warp = threadIdx.x >> 5, pg = (threadIdx.x & 31) >> 2;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    pix[k] = warp * 32 + k * 8 + pg;
-    m[k] = (pix[k] / TS + 1) * TP + pix[k] % TS + 1;
-  }
-}
-
-// forward: out = ReLU(b + conv(in)); the last layer also I = bp + wp . out
-__global__ void __launch_bounds__(TS * TS)
-conv16_fwd(const float* __restrict__ in, int C, int H, int W, const float* __restrict__ w,
-           const float* __restrict__ b, float* __restrict__ out, const float* __restrict__ wp,
-           const float* __restrict__ bp, float* __restrict__ I) {
-  __shared__ __align__(16) float sx[TP * TP * CP];
-  __shared__ __align__(16) float sw[9 * CP * CP];    // [t][ci][co]
-  __shared__ __align__(16) float sb[CP], swp[CP];
-  const int n = blockIdx.z, x0 = blockIdx.x * TS, y0 = blockIdx.y * TS;
-  const int64_t hw = (int64_t)H * W;
-  for (int i = threadIdx.x; i < 9 * CP * CP; i += TS * TS) {
-    const int co = i % CP, ci = (i / CP) % CP, t = i / (CP * CP);
-    sw[i] = (co < C && ci < C) ? w[(co * C + ci) * 9 + t] : 0.0f;
-  }
-  if (threadIdx.x < CP) {
-    sb[threadIdx.x] = threadIdx.x < C ? b[threadIdx.x] : 0.0f;
-    swp[threadIdx.x] = (I && threadIdx.x < C) ? wp[threadIdx.x] : 0.0f;
-  }
-  stage(sx, in + (int64_t)n * C * hw, C, H, W, x0, y0, 1, TP, TP);
-  __syncthreads();
-  const int cg = threadIdx.x & 3;
-  int pix[4], m[4];
-  tile_positions(pix, m);
-  float acc[4][4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[k][c] = sb[4 * cg + c];
-  conv_block(sx, sw, m, cg, acc);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int x = x0 + pix[k] % TS, y = y0 + pix[k] / TS;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      acc[k][c] = fmaxf(acc[k][c], 0.0f);
-      if (x < W && y < H && 4 * cg + c < C)
-        out[((int64_t)n * C + 4 * cg + c) * hw + (int64_t)y * W + x] = acc[k][c];
-    }
-  }
-  if (I) {
-    // Eq. 6: the 4 channel lanes of a position sum their parts; lane cg writes position cg
-    float mine = 0.0f;
-    int pmine = 0;
+  // weights [co][ci][t] -> [t][from][to], zero beyond C: a warp reads runs of 4 x 9 words
+  {
+    float v[4][9];
+    int at[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      float s = swp[4 * cg] * acc[k][0];
-      s = fmaf(swp[4 * cg + 1], acc[k][1], s);
-      s = fmaf(swp[4 * cg + 2], acc[k][2], s);
-      s = fmaf(swp[4 * cg + 3], acc[k][3], s);
-      s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
-      s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
-      if (k == cg) { mine = s; pmine = pix[k]; }
+      const int e = tid + 64 * k, co = (e & 7) + (e >> 2 & 8), ci = (e >> 3 & 3) + (e >> 4 & 12);
+      const bool ok = co < C && ci < C;
+      at[k] = kBwd ? co * CP + ci : ci * CP + co;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) v[k][t] = ok ? w[(co * C + ci) * 9 + t] : 0.0f;
     }
-    const int x = x0 + pmine % TS, y = y0 + pmine / TS;
-    if (x < W && y < H) I[(int64_t)n * hw + (int64_t)y * W + x] = bp[0] + mine;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int t = 0; t < 9; ++t) sw[(kBwd ? 8 - t : t) * kWTap + at[k]] = v[k][t];
+  }
+  const int c0 = warp * 8, x = x0 + lane, y = y0;
+  const int nr = x < W ? H - y : 0;                 // the lane's rows inside the image
+  const int64_t o = ((int64_t)n * C + c0) * hw + (int64_t)y * W + x;
+  if (kBwd)                                         // mask > 0, bit 8 (channel % 4) + row
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float m[4][kRows];
+      uint32_t bits = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+          m[j][r] = r < nr && c0 + 4 * q + j < C ? mask[o + (4 * q + j) * hw + r * W] : 0.0f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) bits |= (m[j][r] > 0.0f ? 1u : 0u) << (8 * j + r);
+      son[q][tid] = bits;
+    }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+
+  f32x2 acc[kRows / 2][8];                          // [row pair][channel]
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const float bc = !kBwd && c0 + c < C ? b[c0 + c] : 0.0f;
+#pragma unroll
+    for (int r = 0; r < kRows / 2; ++r) acc[r][c] = pack2f(bc, bc);
+  }
+#pragma unroll 1
+  for (int t = 0; t < 9; ++t) {
+    const float* xt = sx + t / 3 * kPitch + lane + t % 3;
+    const float* wt = sw + t * kWTap + c0;
+#pragma unroll
+    for (int ci = 0; ci < CP; ++ci) {
+      const float4 wa = *reinterpret_cast<const float4*>(wt + ci * CP);
+      const float4 wb = *reinterpret_cast<const float4*>(wt + ci * CP + 4);
+      const float wc[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+      f32x2 v[kRows / 2];
+#pragma unroll
+      for (int r = 0; r < kRows / 2; ++r)
+        v[r] = pack2f(xt[ci * kPlane + 2 * r * kPitch], xt[ci * kPlane + (2 * r + 1) * kPitch]);
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+#pragma unroll
+        for (int r = 0; r < kRows / 2; ++r) acc[r][c] = fma2(pack2f(wc[c], wc[c]), v[r], acc[r][c]);
+    }
+  }
+  float pI[kRows], p4[kRows];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {                     // four channels at a time
+    float a[4][kRows];
+    const uint32_t on = kBwd ? son[q][tid] : 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int r = 0; r < kRows / 2; ++r) unpack2f(acc[r][4 * q + j], a[j][2 * r], a[j][2 * r + 1]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool okc = c0 + 4 * q + j < C;
+      // Eq. 6 with sums of four channels, then (s0 + s1) + (s2 + s3)
+      const float wq = !kBwd && I && okc ? wp[c0 + 4 * q + j] : 0.0f;
+#pragma unroll
+      for (int r = 0; r < kRows; ++r) {
+        const float v = kBwd ? (on >> (8 * j + r) & 1u ? a[j][r] : 0.0f) : fmaxf(a[j][r], 0.0f);
+        if (okc && r < nr) out[o + (4 * q + j) * hw + r * W] = v;
+        if (!kBwd) p4[r] = j == 0 ? wq * v : fmaf(wq, v, p4[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) pI[r] = q == 0 ? p4[r] : pI[r] + p4[r];
+  }
+  if (!kBwd && I) {
+    __syncthreads();               // every warp is done with sx
+    if (c0)
+#pragma unroll
+      for (int r = 0; r < kRows; ++r) sx[r * CW + lane] = pI[r];
+    __syncthreads();
+    if (!c0)
+#pragma unroll
+      for (int r = 0; r < kRows; ++r)
+        if (r < nr)
+          I[(int64_t)n * hw + (int64_t)(y + r) * W + x] = bp[0] + (pI[r] + sx[r * CW + lane]);
   }
 }
 
-// data backward: dzp[ci] = (sum_co,t w[co][ci][t] dz[co] at the mirrored tap) 1(a_prev > 0),
-// i.e. the forward block with weights w'[t][co][ci] = w[co][ci][8 - t]
-__global__ void __launch_bounds__(TS * TS)
-conv16_bwd_data(const float* __restrict__ dz, int C, int H, int W, const float* __restrict__ w,
-                const float* __restrict__ a_prev, float* __restrict__ dzp) {
-  __shared__ __align__(16) float sx[TP * TP * CP];
-  __shared__ __align__(16) float sw[9 * CP * CP];    // [t][co][ci]
-  const int n = blockIdx.z, x0 = blockIdx.x * TS, y0 = blockIdx.y * TS;
-  const int64_t hw = (int64_t)H * W;
-  for (int i = threadIdx.x; i < 9 * CP * CP; i += TS * TS) {
-    const int ci = i % CP, co = (i / CP) % CP, t = i / (CP * CP);
-    sw[i] = (co < C && ci < C) ? w[(co * C + ci) * 9 + (8 - t)] : 0.0f;
-  }
-  stage(sx, dz + (int64_t)n * C * hw, C, H, W, x0, y0, 1, TP, TP);
-  __syncthreads();
-  const int cg = threadIdx.x & 3;
-  int pix[4], m[4];
-  tile_positions(pix, m);
-  float acc[4][4] = {};
-  conv_block(sx, sw, m, cg, acc);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int x = x0 + pix[k] % TS, y = y0 + pix[k] / TS;
-    if (x >= W || y >= H) continue;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      if (4 * cg + c >= C) continue;
-      const int64_t o = ((int64_t)n * C + 4 * cg + c) * hw + (int64_t)y * W + x;
-      dzp[o] = a_prev[o] > 0.0f ? acc[k][c] : 0.0f;
-    }
-  }
+dim3 conv16_grid(int H, int W, int N) {
+  return dim3((unsigned)((int64_t)((W + CW - 1) / CW) * ((H + kRows - 1) / kRows)), 1, N);
 }
 
 // weight backward: grad w[co][ci][t] += sum_n,p dz[n][co][p] in[n][ci][p + off(t)],
-// grad b[co] += sum dz.  Persistent blocks of 160 threads: thread e < 144 owns
-// (tap t = e / 16, output quad e % 4, input quad (e / 4) % 4), 16 sums; threads
-// 144..159 own the bias sums of one output channel each.  One atomic per entry
-// per block at the end.
-constexpr int kWThreads = 160;
-__global__ void __launch_bounds__(kWThreads)
+// grad b[co] += sum dz.  Persistent blocks over tiles of 8 rows x 32 columns, staged
+// channel-interleaved (16 floats per position, its four 16-byte groups permuted by
+// the column so that staging stores and reads are free of bank conflicts).  Warp
+// (ky, row pair), half-warp = one row, lane = (output quad, input quad): it walks the
+// row's 32 positions with the last three input quads in registers and sums 4 x 4
+// channels for the three taps of row ky: two 16-byte loads per 48 multiply-adds (8
+// clk of shared memory for 12 of the FP32 pipe; a thread per tap and quads, without
+// the window, had 8 for 4 and one block's 256 positions in one chain).  Sums stay
+// in registers until the block's last tile; one atomic per entry and block then.
+// Average launch over the pass above: 97 -> 31 us.  Staging by 4-byte cp.async into two
+// buffers was slower (33 us; 38 with plain channel planes read 4 bytes at a time).
+constexpr int kWRows = 8;
+constexpr int kWThreads = 3 * (kWRows / 2) * 32;
+
+__global__ void __launch_bounds__(kWThreads, 2)
 conv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, int N, int C, int H,
                   int W, float* __restrict__ gw, float* __restrict__ gb) {
-  __shared__ __align__(16) float sd[TS * TS * CP];
-  __shared__ __align__(16) float sx[TP * TP * CP];
-  const int e = threadIdx.x;
-  const int t = e / 16, cq = e % 4, iq = (e / 4) % 4;
-  const int toff = (t / 3) * TP + t % 3;          // tap offset from the tile position's halo corner
-  float acc[4][4] = {};
-  float bsum = 0.0f;
+  constexpr int kWarps = kWThreads / 32, kXRows = kWRows + 2;
+  constexpr int kPart = 9 * CP * CP;              // a row pair's sums
+  __shared__ __align__(16) float sh[(kWRows * CW + kXRows * kPitch) * CP];
+  __shared__ float sb[kWarps][4];
+  static_assert(kWRows / 2 * kPart <= (kWRows * CW + kXRows * kPitch) * CP, "the sums fit the tiles' place");
+  float* const sd = sh;
+  float* const sx = sh + kWRows * CW * CP;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ky = warp % 3, row = warp / 3 * 2 + (lane >> 4), cq = lane & 3, iq = (lane >> 2) & 3;
+  const int g = warp & 3;                         // the channel quad this warp stages (kWarps % 4 == 0)
+  static_assert(kWarps % 4 == 0, "a warp stages one channel quad");
   const int64_t hw = (int64_t)H * W;
-  const int tiles_x = (W + TS - 1) / TS, tiles_y = (H + TS - 1) / TS;
+  const int tiles_x = (W + CW - 1) / CW, tiles_y = (H + kWRows - 1) / kWRows;
   const int64_t ntiles = (int64_t)N * tiles_x * tiles_y;
+  const auto slot = [](int col, int q) { return col * CP + 4 * (q ^ ((col >> 1) & 3)); };
+  f32x2 acc[3][4][2] = {};                        // [kx][output channel][input channel pair]
+  float bs[4] = {};
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int n = (int)(tile / (tiles_x * tiles_y));
     const int tt = (int)(tile % (tiles_x * tiles_y));
-    const int x0 = (tt % tiles_x) * TS, y0 = (tt / tiles_x) * TS;
-    __syncthreads();
-    stage(sd, dz + (int64_t)n * C * hw, C, H, W, x0, y0, 0, TS, TS);
-    stage(sx, in + (int64_t)n * C * hw, C, H, W, x0, y0, 1, TP, TP);
-    __syncthreads();
-    if (e < 144) {
-#pragma unroll 2
-      for (int py = 0; py < TS; ++py) {
-#pragma unroll 4
-        for (int px = 0; px < TS; ++px) {
-          const int p = py * TS + px, q = py * TP + px + toff;
-          const float4 d = *reinterpret_cast<const float4*>(sd + cidx(p, cq));
-          const float4 x = *reinterpret_cast<const float4*>(sx + cidx(q, iq));
-          const float dv[4] = {d.x, d.y, d.z, d.w}, xv[4] = {x.x, x.y, x.z, x.w};
+    const int x0 = (tt % tiles_x) * CW, y0 = (tt / tiles_x) * kWRows;
+    const float* dn = dz + ((int64_t)n * C + 4 * g) * hw;
+    const float* xn = in + ((int64_t)n * C + 4 * g) * hw;
+    float vd[kWRows * 4 / kWarps + 1][4];
 #pragma unroll
-          for (int a = 0; a < 4; ++a)
+    for (int k = 0; k < kWRows * 4 / kWarps + 1; ++k) {
+      const int r = (warp + k * kWarps) >> 2, yy = y0 + r, xx = x0 + lane;
+      const bool ok = r < kWRows && yy < H && xx < W;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][c] = fmaf(dv[a], xv[c], acc[a][c]);
-        }
+      for (int j = 0; j < 4; ++j) vd[k][j] = ok && 4 * g + j < C ? dn[j * hw + (int64_t)yy * W + xx] : 0.0f;
+    }
+    __syncthreads();                              // the last tile's reads
+#pragma unroll
+    for (int k = 0; k < kWRows * 4 / kWarps + 1; ++k) {
+      const int r = (warp + k * kWarps) >> 2;
+      if (r < kWRows)
+        *reinterpret_cast<float4*>(sd + r * CW * CP + slot(lane, g)) =
+            make_float4(vd[k][0], vd[k][1], vd[k][2], vd[k][3]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) bs[j] += vd[k][j];
+    }
+    float vx[kXRows * 4 / kWarps + 1][4];
+#pragma unroll
+    for (int k = 0; k < kXRows * 4 / kWarps + 1; ++k) {
+      const int r = (warp + k * kWarps) >> 2, yy = y0 - 1 + r, xx = x0 - 1 + lane;
+      const bool ok = r < kXRows && yy >= 0 && yy < H && xx >= 0 && xx < W;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) vx[k][j] = ok && 4 * g + j < C ? xn[j * hw + (int64_t)yy * W + xx] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < kXRows * 4 / kWarps + 1; ++k) {
+      const int r = (warp + k * kWarps) >> 2;
+      if (r < kXRows)
+        *reinterpret_cast<float4*>(sx + r * kPitch * CP + slot(lane, g)) =
+            make_float4(vx[k][0], vx[k][1], vx[k][2], vx[k][3]);
+    }
+    if (tid < kXRows * 8) {                       // the two columns right of the lanes'
+      const int q = tid & 3, col = CW + ((tid >> 2) & 1), r = tid >> 3, yy = y0 - 1 + r, xx = x0 - 1 + col;
+      const bool ok = yy >= 0 && yy < H && xx < W;
+      const float* src = in + ((int64_t)n * C + 4 * q) * hw + (int64_t)yy * W + xx;
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = ok && 4 * q + j < C ? src[j * hw] : 0.0f;
+      *reinterpret_cast<float4*>(sx + r * kPitch * CP + slot(col, q)) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    __syncthreads();
+    if (y0 + row < H) {
+      const float* dr = sd + row * CW * CP;
+      const float* xr = sx + (row + ky) * kPitch * CP;
+      ulonglong2 win[3];
+      win[0] = *reinterpret_cast<const ulonglong2*>(xr + slot(0, iq));
+      win[1] = *reinterpret_cast<const ulonglong2*>(xr + slot(1, iq));
+#pragma unroll
+      for (int p = 0; p < CW; ++p) {
+        win[(p + 2) % 3] = *reinterpret_cast<const ulonglong2*>(xr + slot(p + 2, iq));
+        const float4 d = *reinterpret_cast<const float4*>(dr + slot(p, cq));
+        const f32x2 d2[4] = {pack2f(d.x, d.x), pack2f(d.y, d.y), pack2f(d.z, d.z), pack2f(d.w, d.w)};
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            acc[kx][j][0] = fma2(d2[j], win[(p + kx) % 3].x, acc[kx][j][0]);
+            acc[kx][j][1] = fma2(d2[j], win[(p + kx) % 3].y, acc[kx][j][1]);
+          }
       }
-    } else {
-      const int co = e - 144;
-      for (int p = 0; p < TS * TS; ++p) bsum += sd[cidx(p, co >> 2) + (co & 3)];
     }
   }
-  if (e < 144) {
+  // the block's sums: a warp's two rows by shuffle, the four row pairs in shared memory
+  __syncthreads();
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+  for (int kx = 0; kx < 3; ++kx)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int co = 4 * cq + a, ci = 4 * iq + c;
-        if (co < C && ci < C) atomicAdd(gw + (co * C + ci) * 9 + t, acc[a][c]);
-      }
-  } else if (e - 144 < C) {
-    atomicAdd(gb + (e - 144), bsum);
+    for (int j = 0; j < 4; ++j) {
+      float v[4];
+      unpack2f(acc[kx][j][0], v[0], v[1]);
+      unpack2f(acc[kx][j][1], v[2], v[3]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] += __shfl_xor_sync(0xFFFFFFFFu, v[e], 16);
+      if (lane < 16)
+        *reinterpret_cast<float4*>(sh + (((warp / 3 * 3 + kx) * 4 + j) * 48 + ky * 16 + lane) * 4) =
+            make_float4(v[0], v[1], v[2], v[3]);
+    }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) bs[j] += __shfl_xor_sync(0xFFFFFFFFu, bs[j], o);
+    if (lane == 0) sb[warp][j] = bs[j];
   }
+  __syncthreads();
+  for (int i = tid; i < 9 * C * C; i += kWThreads) {
+    const int t = i % 9, ci = i / 9 % C, co = i / 9 / C;
+    const float* s = sh + (((t % 3) * 4 + (co & 3)) * 48 + t / 3 * 16 + (ci >> 2) * 4 + (co >> 2)) * 4 + (ci & 3);
+    atomicAdd(gw + i, (s[0] + s[kPart]) + (s[2 * kPart] + s[3 * kPart]));
+  }
+  if (tid < C) atomicAdd(gb + tid, (sb[tid >> 2][tid & 3] + sb[(tid >> 2) + 4][tid & 3]) + sb[(tid >> 2) + 8][tid & 3]);
 }
 
 // ------------------------------------------------------------ loss (Eq. 7-11)
@@ -622,7 +706,7 @@ int seg_forward(const float* logl, const et_train_shape* sh, const et_evsnet_wei
                 const Workspace& ws, int k0, int nseg, cudaStream_t st) {
   const int H = sh->H, W = sh->W, C = net->C, L = net->n_layers;
   const int N = sh->B * nseg;
-  dim3 grid((W + TS - 1) / TS, (H + TS - 1) / TS, N);
+  const dim3 grid((W + TS - 1) / TS, (H + TS - 1) / TS, N), grid16 = conv16_grid(H, W, N);
   const float* wproj = net->w + wofs(L, C);
   const float* bproj = net->b + (int64_t)L * C;
   for (int l = 0; l < L; ++l) {
@@ -636,9 +720,9 @@ int seg_forward(const float* logl, const et_train_shape* sh, const et_evsnet_wei
                                       last ? ws.I : nullptr, nullptr, false, st);
       if (rc != ET_OK) return rc;
     } else
-      conv16_fwd<<<grid, TS * TS, 0, st>>>(ws.act[l - 1], C, H, W, net->w + wofs(l, C),
-                                           net->b + (int64_t)l * C, ws.act[l], wproj, bproj,
-                                           last ? ws.I : nullptr);
+      conv16<false><<<grid16, 64, 0, st>>>(ws.act[l - 1], C, H, W, net->w + wofs(l, C),
+                                            net->b + (int64_t)l * C, ws.act[l], wproj, bproj,
+                                            last ? ws.I : nullptr, nullptr);
     ET_CHECK_LAUNCH();
   }
   return ET_OK;
@@ -752,7 +836,7 @@ extern "C" int et_evsnet_train_backward(const float* logl, const et_train_shape*
     proj_bwd<<<nsm * 4, 256, 0, st>>>(ws.dI, ws.act[L - 1], N, C, hw, net->w + wofs(L, C), ws.dz[0],
                                       gwp, gbp);
     ET_CHECK_LAUNCH();
-    dim3 grid((W + TS - 1) / TS, (H + TS - 1) / TS, N);
+    const dim3 grid16 = conv16_grid(H, W, N);
     int cur = 0;
     for (int l = L - 1; l >= 0; --l) {
       if (l == 0)
@@ -772,8 +856,8 @@ extern "C" int et_evsnet_train_backward(const float* logl, const et_train_shape*
                                 nullptr, nullptr, nullptr, ws.act[l - 1], true, st);
           if (rc != ET_OK) return rc;
         } else {
-          conv16_bwd_data<<<grid, TS * TS, 0, st>>>(ws.dz[cur], C, H, W, net->w + wofs(l, C),
-                                                    ws.act[l - 1], ws.dz[cur ^ 1]);
+          conv16<true><<<grid16, 64, 0, st>>>(ws.dz[cur], C, H, W, net->w + wofs(l, C), nullptr, ws.dz[cur ^ 1],
+                                               nullptr, nullptr, nullptr, ws.act[l - 1]);
           ET_CHECK_LAUNCH();
         }
         cur ^= 1;
