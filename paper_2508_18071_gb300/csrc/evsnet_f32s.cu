@@ -3,24 +3,32 @@
 // 16 channels, the point-wise projection (Eq. 6) and BiLIF (Eq. 2-3).
 //
 // Each CTA owns a 32 x 16 pixel tile for the whole call and walks the frames;
-// the membrane potentials of its pixels stay in shared memory.  Per step the
+// the membrane potentials of its pixels stay in registers.  Per step the
 // log frame tile with an L-pixel halo is loaded (X = l_k - l_{k-1}, Eq. 1) and
 // the layers run one after the other on shrinking regions of the padded tile
 // (layer l is computed L - 1 - l pixels beyond the tile), with zero padding
 // outside the image.
 //
-// Activations are stored channel-interleaved in shared memory, 16 floats per
-// position, the four 16-byte channel groups of position m permuted by
-// ((m >> 1) & 3) so that eight consecutive positions read one group from eight
-// different bank quads.  In layers 1.. a thread computes 4 output channels for
-// 4 positions: per tap and group of 4 input channels it loads 4 weight vectors
-// (shared by the 8 position lanes of its channel group) and 4 activation
-// vectors (shared by the 4 channel lanes of its position) for 64 FMAs.  In the
-// last layer the 4 channel lanes of a position sum their parts of the
-// projection with two shuffles and each takes one position for BiLIF.
+// What bounds it is shared memory: a warp's 16-byte load takes 4 clk of the SM's
+// 128 bytes per clk whatever its addresses.  In layers 1.. a lane computes 8 output
+// channels for 4 to 8 positions, as many as spread the layer's region over the CTA's
+// eight warps: 8 weight loads and one per position feed 32 multiply-adds per position
+// (48 to 64 clk of shared memory for 32 to 64 of the FP32 pipe; 4 positions x 4
+// channels, 32 clk for 16, kept shared memory 97 % busy).  Multiply-adds run as FP32
+// pairs over channels, rounded like fmaf, in one chain over taps, then input channels.
+// Activations lie by groups of four channels, [group][position]: consecutive positions
+// are consecutive 16-byte words.  A layer's outputs stay in registers until every warp
+// has read its inputs and then replace them, so that one activation buffer serves all
+// layers and two CTAs fit an SM at four layers.  In the last layer the two channel
+// lanes of a position add their parts of the projection and each takes two rows of one
+// column for BiLIF; events are gathered per warp.  641 x 363, four layers, 15 steps:
+// 2.35 -> 1.66 ms (2.10 with 8 positions everywhere: six, five and four of the warps
+// then have work).
 #include "et_internal.cuh"
 #include "event_emit.cuh"
 #include "evsnet_common.h"
+#include "f32x2.cuh"
+#include <type_traits>
 
 namespace {
 
@@ -32,35 +40,78 @@ struct SParams {
   float beta, vth, reset;
   int H, W, F, f0, t0;
   int Wp, Hp;
-  int off_act1, off_b, off_w0, off_wl, off_wp, off_cur, off_prev, off_V;
+  int plane;                      // floats of one channel group's activations
+  int off_b, off_w0, off_wl, off_wp, off_cur, off_prev;
 };
 
-__device__ __forceinline__ int act_idx(int m, int g) { return m * CP + 4 * (g ^ ((m >> 1) & 3)); }
+constexpr int kWarps = 8;         // of a CTA; a warp's 16 position lanes x 2 channel lanes
+constexpr int kThreads = kWarps * 32;
+constexpr int kLastPos = TW * TH / (kWarps * 16);   // a lane's positions in the last layer
+constexpr int kLastRows = kLastPos / 2;
+static_assert(TW == 32 && kLastPos == 2 * kLastRows, "a lane of the last layer owns rows of one column");
+constexpr int kStageCap = 64;    // events a warp holds before it appends them
 
 __device__ __forceinline__ float4 relu4(float a, float b, float c, float d) {
   return make_float4(fmaxf(a, 0.0f), fmaxf(b, 0.0f), fmaxf(c, 0.0f), fmaxf(d, 0.0f));
 }
 
-template <int kThreads>
-__global__ void __launch_bounds__(kThreads)
+// one 3x3 layer: sums of kP positions (words at[k] of act's first group) x the channels
+// 8 cg .. whose weights start at wt, from the biases b
+template <int kP>
+__device__ __forceinline__ void conv_layer(const float* act, int plane, int Wp, const float* wt, const float* b,
+                                           const int (&at)[kP], f32x2 (&acc)[kP][4]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const f32x2 b2 = *reinterpret_cast<const f32x2*>(b + 2 * c);
+#pragma unroll
+    for (int k = 0; k < kP; ++k) acc[k][c] = b2;
+  }
+#pragma unroll 1
+  for (int t = 0; t < 9; ++t) {
+    const float* xt = act + 4 * ((t / 3 - 1) * Wp + t % 3 - 1);
+#pragma unroll
+    for (int g = 0; g < CP / 4; ++g, wt += 4 * CP, xt += plane) {
+      ulonglong2 w[4][2];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        w[c][0] = *reinterpret_cast<const ulonglong2*>(wt + c * CP);
+        w[c][1] = *reinterpret_cast<const ulonglong2*>(wt + c * CP + 4);
+      }
+#pragma unroll
+      for (int k = 0; k < kP; ++k) {
+        const float4 x = *reinterpret_cast<const float4*>(xt + at[k]);
+        const float xc[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const f32x2 x2 = pack2f(xc[c], xc[c]);
+          acc[k][0] = fma2(w[c][0].x, x2, acc[k][0]);
+          acc[k][1] = fma2(w[c][0].y, x2, acc[k][1]);
+          acc[k][2] = fma2(w[c][1].x, x2, acc[k][2]);
+          acc[k][3] = fma2(w[c][1].y, x2, acc[k][3]);
+        }
+      }
+    }
+  }
+}
+
+template <int kBlocks>
+__global__ void __launch_bounds__(kThreads, kBlocks)
 evsnet_f32s_kernel(SParams P, int C, const float* __restrict__ logl, const float* __restrict__ wg,
                    const float* __restrict__ bg, float* __restrict__ Vg,
                    const float* __restrict__ last_l, et_event* events, int64_t cap,
                    unsigned long long* n_events, float* __restrict__ I_out,
                    int8_t* __restrict__ spikes) {
   extern __shared__ __align__(16) float sm[];
+  __shared__ uint32_t staged[kWarps][kStageCap];
   const int L = P.L, Wp = P.Wp, Hp = P.Hp, tid = threadIdx.x;
-  constexpr int kWarps = kThreads / 32;
-  const int warp = tid >> 5, lane = tid & 31, pg = lane >> 2, cg = lane & 3;
-  float* const act0 = sm;                         // [Hp Wp][CP], permuted groups
-  float* const act1 = sm + P.off_act1;
+  const int warp = tid >> 5, lane = tid & 31, pg = lane >> 1, cg = lane & 1;
+  float* const act = sm;                          // [CP / 4][Hp Wp][4]
   float* const sb = sm + P.off_b;                 // [L][CP] biases, then the projection bias
   float* const w0 = sm + P.off_w0;                // [9][CP]
   float* const wl = sm + P.off_wl;                // [L-1][9][CP (ci)][CP (co)]
   float* const wp = sm + P.off_wp;                // [CP]
   float* cur = sm + P.off_cur;                    // log frame over the padded tile
   float* prev = sm + P.off_prev;
-  float* const Vs = sm + P.off_V;                 // [TH][TW]
   const int tiles_x = (P.W + TW - 1) / TW;
   const int ox = (blockIdx.x % tiles_x) * TW, oy = (blockIdx.x / tiles_x) * TH;
   const int64_t npix = (int64_t)P.H * P.W;
@@ -80,10 +131,13 @@ evsnet_f32s_kernel(SParams P, int C, const float* __restrict__ logl, const float
   }
   for (int i = tid; i < CP; i += kThreads) wp[i] = i < C ? wg[9 * C + (L - 1) * C * C * 9 + i] : 0.0f;
   if (tid == 0) sb[L * CP] = bg[L * C];
-  for (int i = tid; i < TW * TH; i += kThreads) {
-    const int gx = ox + i % TW, gy = oy + i / TW;
-    Vs[i] = (gx < P.W && gy < P.H) ? Vg[(int64_t)gy * P.W + gx] : 0.0f;
-  }
+  // the lane's pixels in the last layer: column vx, rows vy ..
+  const int vx = ox + 16 * cg + pg, vy = oy + kLastRows * warp;
+  float V[kLastRows];
+#pragma unroll
+  for (int j = 0; j < kLastRows; ++j)
+    V[j] = vx < P.W && vy + j < P.H ? Vg[(int64_t)(vy + j) * P.W + vx] : 0.0f;
+  EventStage<kStageCap> stage(staged[warp], events, cap, n_events, (uint32_t)vx, (uint32_t)vy, (uint32_t)P.t0);
   // the frame before the first step: the caller's last frame, or frame 0 when
   // the state is fresh (the first step is then frame 1)
   for (int i = tid; i < Hp * Wp; i += kThreads) {
@@ -102,157 +156,149 @@ evsnet_f32s_kernel(SParams P, int C, const float* __restrict__ logl, const float
     }
     __syncthreads();
     // layer 0 (one input channel) on rows / columns [1, Hp - 1) x [1, Wp - 1):
-    // one thread per position, all channels
+    // two positions per thread, all channels
     {
-      const int rw = Wp - 2;
-      for (int i = tid; i < (Hp - 2) * rw; i += kThreads) {
-        const int py = 1 + i / rw, px = 1 + i % rw, m = py * Wp + px;
-        const int gx = ox - L + px, gy = oy - L + py;
-        float acc[CP];
+      const int rw = Wp - 2, n = (Hp - 2) * rw;
+      for (int i = tid; i < n; i += 2 * kThreads) {
+        int m[2];
+        bool in[2];
+        f32x2 acc[2][CP / 2];
 #pragma unroll
-        for (int c = 0; c < CP; ++c) acc[c] = sb[c];
-#pragma unroll
-        for (int t = 0; t < 9; ++t) {
-          const int q = m + (t / 3 - 1) * Wp + (t % 3 - 1);
-          const float x = cur[q] - prev[q];                     // Eq. 1
-          const float4* w4 = reinterpret_cast<const float4*>(w0 + t * CP);
-#pragma unroll
-          for (int j = 0; j < CP / 4; ++j) {
-            const float4 w = w4[j];
-            acc[4 * j] = fmaf(w.x, x, acc[4 * j]);
-            acc[4 * j + 1] = fmaf(w.y, x, acc[4 * j + 1]);
-            acc[4 * j + 2] = fmaf(w.z, x, acc[4 * j + 2]);
-            acc[4 * j + 3] = fmaf(w.w, x, acc[4 * j + 3]);
-          }
-        }
-        const bool in = gx >= 0 && gx < P.W && gy >= 0 && gy < P.H;
-#pragma unroll
-        for (int j = 0; j < CP / 4; ++j)
-          *reinterpret_cast<float4*>(act0 + act_idx(m, j)) =
-              in ? relu4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3])
-                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      }
-    }
-    __syncthreads();
-    // layers 1 .. L-1; the last one only on the tile, into projection + BiLIF
-    for (int l = 1; l < L; ++l) {
-      const float* ain = (l & 1) ? act0 : act1;
-      float* aout = (l & 1) ? act1 : act0;
-      const float* wlay = wl + (l - 1) * 9 * CP * CP + 4 * cg;
-      const bool last = l == L - 1;
-      const int r0 = last ? L : l + 1, r1 = last ? L + TH : Hp - l - 1;
-      const int c0 = last ? L : l + 1, c1 = last ? L + TW : Wp - l - 1;
-      const int rw = c1 - c0, n = (r1 - r0) * rw;
-      const int nchunks = (n + 31) / 32;
-      // warp-uniform chunks of 32 positions: position k of lane (pg, cg) is
-      // chunk * 32 + k * 8 + pg
-      for (int j = warp; j < nchunks; j += kWarps) {
-        int m[4];
-        bool st[4], in[4];
-        int gxk[4], gyk[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int idx = j * 32 + k * 8 + pg;
-          st[k] = idx < n;
-          const int ic = st[k] ? idx : n - 1;
-          const int py = r0 + ic / rw, px = c0 + ic % rw;
+        for (int k = 0; k < 2; ++k) {
+          const int ic = min(i + k * kThreads, n - 1), py = 1 + ic / rw, px = 1 + ic % rw;
+          const int gx = ox - L + px, gy = oy - L + py;
           m[k] = py * Wp + px;
-          gxk[k] = ox - L + px; gyk[k] = oy - L + py;
-          in[k] = st[k] && gxk[k] >= 0 && gxk[k] < P.W && gyk[k] >= 0 && gyk[k] < P.H;
+          in[k] = gx >= 0 && gx < P.W && gy >= 0 && gy < P.H;
+#pragma unroll
+          for (int c = 0; c < CP / 2; ++c) acc[k][c] = *reinterpret_cast<const f32x2*>(sb + 2 * c);
         }
-        float acc[4][4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[k][c] = sb[l * CP + 4 * cg + c];
-#pragma unroll 3
         for (int t = 0; t < 9; ++t) {
-          const int toff = (t / 3 - 1) * Wp + (t % 3 - 1);
-          const float* wt = wlay + t * CP * CP;
-          int mk[4];
+          f32x2 x[2];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) mk[k] = m[k] + toff;
+          for (int k = 0; k < 2; ++k) {
+            const int q = m[k] + (t / 3 - 1) * Wp + (t % 3 - 1);
+            const float v = cur[q] - prev[q];                   // Eq. 1
+            x[k] = pack2f(v, v);
+          }
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const float4 wa = *reinterpret_cast<const float4*>(wt + (4 * g + 0) * CP);
-            const float4 wb = *reinterpret_cast<const float4*>(wt + (4 * g + 1) * CP);
-            const float4 wc = *reinterpret_cast<const float4*>(wt + (4 * g + 2) * CP);
-            const float4 wd = *reinterpret_cast<const float4*>(wt + (4 * g + 3) * CP);
+          for (int c = 0; c < CP / 2; c += 2) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(w0 + t * CP + 2 * c);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float4 x = *reinterpret_cast<const float4*>(ain + act_idx(mk[k], g));
-              acc[k][0] = fmaf(wa.x, x.x, acc[k][0]);
-              acc[k][1] = fmaf(wa.y, x.x, acc[k][1]);
-              acc[k][2] = fmaf(wa.z, x.x, acc[k][2]);
-              acc[k][3] = fmaf(wa.w, x.x, acc[k][3]);
-              acc[k][0] = fmaf(wb.x, x.y, acc[k][0]);
-              acc[k][1] = fmaf(wb.y, x.y, acc[k][1]);
-              acc[k][2] = fmaf(wb.z, x.y, acc[k][2]);
-              acc[k][3] = fmaf(wb.w, x.y, acc[k][3]);
-              acc[k][0] = fmaf(wc.x, x.z, acc[k][0]);
-              acc[k][1] = fmaf(wc.y, x.z, acc[k][1]);
-              acc[k][2] = fmaf(wc.z, x.z, acc[k][2]);
-              acc[k][3] = fmaf(wc.w, x.z, acc[k][3]);
-              acc[k][0] = fmaf(wd.x, x.w, acc[k][0]);
-              acc[k][1] = fmaf(wd.y, x.w, acc[k][1]);
-              acc[k][2] = fmaf(wd.z, x.w, acc[k][2]);
-              acc[k][3] = fmaf(wd.w, x.w, acc[k][3]);
+            for (int k = 0; k < 2; ++k) {
+              acc[k][c] = fma2(w.x, x[k], acc[k][c]);
+              acc[k][c + 1] = fma2(w.y, x[k], acc[k][c + 1]);
             }
           }
         }
-        if (!last) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (st[k])
-              *reinterpret_cast<float4*>(aout + act_idx(m[k], cg)) =
-                  in[k] ? relu4(acc[k][0], acc[k][1], acc[k][2], acc[k][3])
-                        : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        } else {
-          // Eq. 6: each channel lane's part of the projection, summed over the
-          // 4 lanes of the position (the same sum in every lane)
-          const float4 wpv = *reinterpret_cast<const float4*>(wp + 4 * cg);
-          float Ik[4];
+        for (int k = 0; k < 2; ++k) {
+          if (i + k * kThreads >= n) break;
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            float s = wpv.x * fmaxf(acc[k][0], 0.0f);
-            s = fmaf(wpv.y, fmaxf(acc[k][1], 0.0f), s);
-            s = fmaf(wpv.z, fmaxf(acc[k][2], 0.0f), s);
-            s = fmaf(wpv.w, fmaxf(acc[k][3], 0.0f), s);
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            s += __shfl_xor_sync(0xffffffffu, s, 2);
-            Ik[k] = sb[L * CP] + s;
+          for (int g = 0; g < CP / 4; ++g) {
+            float a[4];
+            unpack2f(acc[k][2 * g], a[0], a[1]);
+            unpack2f(acc[k][2 * g + 1], a[2], a[3]);
+            *reinterpret_cast<float4*>(act + g * P.plane + 4 * m[k]) =
+                in[k] ? relu4(a[0], a[1], a[2], a[3]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
           }
-          // lane cg takes position k = cg
-          float I = Ik[0];
-          int mm = m[0], gx = gxk[0], gy = gyk[0];
-          bool own = in[0];
+        }
+      }
+    }
+    __syncthreads();
+    // layers 1 .. L-2, each on rows / columns [l + 1, ..): position k of lane (pg, cg)
+    // is (k * kWarps + warp) * 16 + pg
+    auto hidden = [&](auto pos, int l) {
+      constexpr int kP = decltype(pos)::value;
+      const int rw = TW + 2 * (L - 1 - l), n = (TH + 2 * (L - 1 - l)) * rw;
+      int at[kP];
+      uint32_t in = 0;                            // positions of the image
 #pragma unroll
-          for (int k = 1; k < 4; ++k)
-            if (cg == k) { I = Ik[k]; mm = m[k]; gx = gxk[k]; gy = gyk[k]; own = in[k]; }
-          uint32_t nev = 0;
-          int S = 0;
-          if (own) {
-            const int ti = (mm / Wp - L) * TW + (mm % Wp - L);
-            const float vp = P.beta * Vs[ti] + I;               // Eq. 2-3
-            S = vp >= P.vth ? 1 : (vp <= -P.vth ? -1 : 0);
-            Vs[ti] = vp - P.reset * (float)S;
-            nev = (S != 0 && P.t0 + f >= 0) ? 1u : 0u;   // delayed labels below 0: none
-            const int64_t o = (int64_t)(f - P.f0) * npix + (int64_t)gy * P.W + gx;
-            if (I_out) I_out[o] = I;
-            if (spikes) spikes[o] = (int8_t)S;
-          }
-          emit_events_warp(events, cap, n_events, nev, (uint32_t)(own ? gx : 0),
-                           (uint32_t)(own ? gy : 0), (uint32_t)(P.t0 + f), S);
+      for (int k = 0; k < kP; ++k) {
+        const int ic = min((k * kWarps + warp) * 16 + pg, n - 1);
+        const int py = l + 1 + ic / rw, px = l + 1 + ic % rw;
+        const int gx = ox - L + px, gy = oy - L + py;
+        at[k] = 4 * (py * Wp + px);
+        in |= (gx >= 0 && gx < P.W && gy >= 0 && gy < P.H ? 1u : 0u) << k;
+      }
+      f32x2 acc[kP][4];
+      conv_layer(act, P.plane, Wp, wl + (l - 1) * 9 * CP * CP + 8 * cg, sb + l * CP + 8 * cg, at, acc);
+      __syncthreads();                            // every warp has read this layer's inputs
+#pragma unroll
+      for (int k = 0; k < kP; ++k) {
+        if ((k * kWarps + warp) * 16 + pg >= n) break;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float a[4];
+          unpack2f(acc[k][2 * h], a[0], a[1]);
+          unpack2f(acc[k][2 * h + 1], a[2], a[3]);
+          *reinterpret_cast<float4*>(act + (2 * cg + h) * P.plane + at[k]) =
+              (in >> k & 1u) ? relu4(a[0], a[1], a[2], a[3]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
       }
       __syncthreads();
+    };
+#pragma unroll 1
+    for (int l = 1; l < L - 1; ++l) {
+      const int per = L - 1 - l;                  // 5, 6, 7, 8 positions of a lane cover its region
+      if (per == 1) hidden(std::integral_constant<int, 5>{}, l);
+      else if (per == 2 || kBlocks == 2) hidden(std::integral_constant<int, 6>{}, l);
+      else if (per == 3) hidden(std::integral_constant<int, 7>{}, l);
+      else hidden(std::integral_constant<int, 8>{}, l);
     }
+    // the last layer on the tile, into projection + BiLIF: a warp owns kLastRows rows
+    {
+      int at[kLastPos];
+#pragma unroll
+      for (int k = 0; k < kLastPos; ++k)
+        at[k] = 4 * ((L + kLastRows * warp + k / 2) * Wp + L + 16 * (k % 2) + pg);
+      f32x2 acc[kLastPos][4];
+      conv_layer(act, P.plane, Wp, wl + (L - 2) * 9 * CP * CP + 8 * cg, sb + (L - 1) * CP + 8 * cg, at, acc);
+      // Eq. 6: sums of four channels, the lane's two, then the other lane's
+      float I[kLastPos];
+#pragma unroll
+      for (int k = 0; k < kLastPos; ++k) {
+        float s[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 wpv = *reinterpret_cast<const float4*>(wp + 8 * cg + 4 * h);
+          float a[4];
+          unpack2f(acc[k][2 * h], a[0], a[1]);
+          unpack2f(acc[k][2 * h + 1], a[2], a[3]);
+          s[h] = wpv.x * fmaxf(a[0], 0.0f);
+          s[h] = fmaf(wpv.y, fmaxf(a[1], 0.0f), s[h]);
+          s[h] = fmaf(wpv.z, fmaxf(a[2], 0.0f), s[h]);
+          s[h] = fmaf(wpv.w, fmaxf(a[3], 0.0f), s[h]);
+        }
+        I[k] = s[0] + s[1];
+        I[k] += __shfl_xor_sync(0xffffffffu, I[k], 1);
+        I[k] = sb[L * CP] + I[k];
+      }
+      // lane cg takes the positions of its column
+      uint32_t fired = 0, neg = 0;
+#pragma unroll
+      for (int j = 0; j < kLastRows; ++j) {
+        const float Ij = cg ? I[2 * j + 1] : I[2 * j];
+        const float vp = P.beta * V[j] + Ij;                    // Eq. 2-3
+        const int S = vp >= P.vth ? 1 : (vp <= -P.vth ? -1 : 0);
+        V[j] = vp - P.reset * (float)S;
+        if (vx >= P.W || vy + j >= P.H) continue;
+        fired |= (S != 0 ? 1u : 0u) << j;
+        neg |= (S < 0 ? 1u : 0u) << j;
+        const int64_t o = (int64_t)(f - P.f0) * npix + (int64_t)(vy + j) * P.W + vx;
+        if (I_out) I_out[o] = Ij;
+        if (spikes) spikes[o] = (int8_t)S;
+      }
+      if (P.t0 + f < 0) fired = 0;                              // delayed labels below 0: none
+      stage.add_rows<kLastRows>(fired, neg, (uint32_t)f, 0);
+    }
+    // the frame loop's barrier after the next frame's load covers the last layer's reads
     float* t = cur; cur = prev; prev = t;
   }
-  for (int i = tid; i < TW * TH; i += kThreads) {
-    const int gx = ox + i % TW, gy = oy + i / TW;
-    if (gx < P.W && gy < P.H) Vg[(int64_t)gy * P.W + gx] = Vs[i];
-  }
+  stage.flush();
+#pragma unroll
+  for (int j = 0; j < kLastRows; ++j)
+    if (vx < P.W && vy + j < P.H) Vg[(int64_t)(vy + j) * P.W + vx] = V[j];
 }
 
 }  // namespace
@@ -268,34 +314,33 @@ int et_evsnet_forward_f32s(const float* logl, int32_t F, const et_evsnet_weights
   P.H = st->H; P.W = st->W; P.F = F; P.f0 = st->initialized ? 0 : 1; P.t0 = t0;
   P.Wp = TW + 2 * P.L; P.Hp = TH + 2 * P.L;
   auto al4 = [](int x) { return (x + 3) & ~3; };           // 16-byte alignment in floats
-  const int act = P.Hp * P.Wp * CP;
-  int off = 2 * act;
-  P.off_act1 = act;
+  // a channel group's activations, an odd multiple of 64 bytes: the two channel lanes
+  // of a position store to different banks
+  P.plane = (P.Hp * P.Wp + 7) / 8 * 32 + 16;
+  int off = CP / 4 * P.plane;
   P.off_b = off; off += al4(P.L * CP + 1);
   P.off_w0 = off; off += 9 * CP;
   P.off_wl = off; off += (P.L - 1) * 9 * CP * CP;
   P.off_wp = off; off += CP;
   P.off_cur = off; off += al4(P.Hp * P.Wp);
   P.off_prev = off; off += al4(P.Hp * P.Wp);
-  P.off_V = off; off += TW * TH;
   const size_t smem = sizeof(float) * (size_t)off;
   int dev = 0, max_smem = 0;
   ET_CHECK_CUDA(cudaGetDevice(&dev));
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (smem > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
-  int sm_smem = 0;
-  ET_CHECK_CUDA(cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-  // one CTA per SM (deep networks: the activation buffers take most of the
-  // shared memory) gets 16 warps to hide the shared-memory latency; two or
-  // more per SM keep 8 warps each (a finer split of the layer regions)
+  // from seven layers on the halo is most of the work: the general kernel takes the call
+  if (P.L > 6) return ET_ERR_UNIMPLEMENTED;
+  // Up to four layers (98 KB, at most 6 positions per lane) two CTAs fit an SM and share
+  // its registers; from five on one has them alone
+  auto kern = P.L <= 4 ? evsnet_f32s_kernel<2> : evsnet_f32s_kernel<1>;
+  cudaFuncAttributes fa;
+  ET_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
+  if (smem + fa.sharedSizeBytes > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
   const int tiles = ((P.W + TW - 1) / TW) * ((P.H + TH - 1) / TH);
-  auto run = [&](auto kern, int threads) -> int {
-    ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<tiles, threads, smem, stream>>>(P, net->C, logl, net->w, net->b, st->V, st->last_l, events, cap,
-                                           reinterpret_cast<unsigned long long*>(n_events), I_out, spikes);
-    ET_CHECK_LAUNCH();
-    return ET_OK;
-  };
-  if (2 * (smem + 1024) > (size_t)sm_smem) return run(evsnet_f32s_kernel<512>, 512);
-  return run(evsnet_f32s_kernel<256>, 256);
+  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<tiles, kThreads, smem, stream>>>(
+      P, net->C, logl, net->w, net->b, st->V, st->last_l, events, cap,
+      reinterpret_cast<unsigned long long*>(n_events), I_out, spikes);
+  ET_CHECK_LAUNCH();
+  return ET_OK;
 }
