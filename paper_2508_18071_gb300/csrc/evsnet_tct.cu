@@ -68,7 +68,7 @@
 // What bounds it: the chain of a round (layer 0's and the epilogues' CUDA-core
 // work between two barriers, ~7 k clk for two steps of 128 pixels against ~1.5 k
 // of MMAs), and per tile reading and writing the FP32 history (20 k and 11 k clk;
-// at 1280x720 3.1 GB a call).  Hence the kernel is compiled per form (no
+// at 1280x720 4.2 GB a call).  Hence the kernel is compiled per form (no
 // runtime choice of stem or input path inside the round), layer 0 and the
 // epilogues run on FP32 pairs (fma.rn.f32x2, bit-identical to fmaf) with 16-byte
 // weight loads, events are gathered per warp, and the history moves a channel row
