@@ -25,6 +25,21 @@ void et_count_launch();
 
 void et_set_last_cuda_error(cudaError_t e);
 
+// Lets launches of `kern` ask for all the shared memory a block can have beside the
+// kernel's static part.  The limit belongs to the function: set to what one launch
+// takes, it could fail another thread's larger launch of the same kernel.
+template <typename K>
+inline int et_allow_shared(K kern) {
+  int dev = 0, per_block = 0;
+  cudaFuncAttributes fa;
+  ET_CHECK_CUDA(cudaGetDevice(&dev));
+  ET_CHECK_CUDA(cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  ET_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
+  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     per_block - (int)fa.sharedSizeBytes));
+  return ET_OK;
+}
+
 // --------------------------------------------------------------- scene layout
 // Triangles are stored in BVH leaf order as three float4: (v0, prim id bits),
 // (v1, material bits), (v2, 0).  Light triangles carry material LIGHT_BIT | light.

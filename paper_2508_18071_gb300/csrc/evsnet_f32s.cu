@@ -337,7 +337,8 @@ int et_evsnet_forward_f32s(const float* logl, int32_t F, const et_evsnet_weights
   ET_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
   if (smem + fa.sharedSizeBytes > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
   const int tiles = ((P.W + TW - 1) / TW) * ((P.H + TH - 1) / TH);
-  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int rc = et_allow_shared(kern);
+  if (rc != ET_OK) return rc;
   kern<<<tiles, kThreads, smem, stream>>>(
       P, net->C, logl, net->w, net->b, st->V, st->last_l, events, cap,
       reinterpret_cast<unsigned long long*>(n_events), I_out, spikes);

@@ -347,7 +347,8 @@ int et_evsnet_forward_pix16(const float* logl, int32_t F, const et_evsnet_weight
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   auto kern = evsnet_pix16_kernel;
   if (smem + sizeof(uint32_t) * kStageCap > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
-  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int rc = et_allow_shared(kern);
+  if (rc != ET_OK) return rc;
   kern<<<(unsigned)std::min<int64_t>(tiles, nsm), kThreads, smem, stream>>>(
       P, logl, net->w, net->b, st->V, st->hist, st->last_l, events, cap,
       reinterpret_cast<unsigned long long*>(n_events), I_out, spikes);

@@ -380,7 +380,8 @@ int et_evsnet_forward_tc16(const float* logl, int32_t F, const et_evsnet_weights
   P.tmem_cols = S * CP <= 64 ? 64 : 128;
   P.wait_iters = et_tc_wait_iters();
   auto kern = S == 4 ? evsnet_tc16_kernel<4> : S == 6 ? evsnet_tc16_kernel<6> : evsnet_tc16_kernel<8>;
-  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const int rc = et_allow_shared(kern);
+  if (rc != ET_OK) return rc;
   kern<<<(unsigned)tiles, kThreads, smem, stream>>>(
       P, logl, net->w, net->b, st->V, st->last_l, events, cap, reinterpret_cast<unsigned long long*>(n_events),
       I_out, spikes);

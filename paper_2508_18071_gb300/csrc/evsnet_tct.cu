@@ -996,7 +996,8 @@ int tct_launch(const float* logl, int32_t F, const et_evsnet_weights* net, et_ev
   ET_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
   if (smem + fa.sharedSizeBytes > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
   if (P.kt > 1 && !st->hist) return ET_ERR_ARG;
-  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int rc = et_allow_shared(kern);
+  if (rc != ET_OK) return rc;
   P.tiles = (int)(((int64_t)P.H * P.W + TP - 1) / TP);
   // one CTA per SM (shared memory, TMEM), each walking tiles: the weights are staged
   // once (a CTA per tile: 400 us more per 1280x720 call)

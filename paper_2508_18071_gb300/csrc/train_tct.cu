@@ -841,7 +841,7 @@ int et_train_tct_conv(const float* in, int B, int K, int64_t hw, int C, int kt, 
     const size_t smem = (size_t)(data_grad ? 1 + 2 + 1 : 2 + 2) * 2 * kBox + (size_t)(kt + 1) * kSlot +
                         (size_t)kt * CP * CP * 2;
     auto kern = data_grad ? tct_conv16<true> : tct_conv16<false>;
-    ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if ((rc = et_allow_shared(kern)) != ET_OK) return rc;
     kern<<<grid, TP, smem, st>>>(m_in, m_extra, m_mask, m_out, A);
     ET_CHECK_LAUNCH();
     return ET_OK;

@@ -1122,7 +1122,7 @@ int launch_conv_tma(bool data_grad, const float* in, int B, int K, int64_t hw, i
   ET_TRY(sm_count(&nsm));
   const int smem = kRing * kBox + kt * 256 * (int)sizeof(float);
   auto kern = data_grad ? tconv16_tma<true> : tconv16_tma<false>;
-  ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ET_TRY(et_allow_shared(kern));
   kern<<<(unsigned)std::min<int64_t>(A.total, nsm), 256, smem, st>>>(m_in, A);
   ET_CHECK_LAUNCH();
   return ET_OK;
