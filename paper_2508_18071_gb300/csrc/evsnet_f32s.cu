@@ -14,8 +14,9 @@
 // channels for 4 to 8 positions, as many as spread the layer's region over the CTA's
 // eight warps: 8 weight loads and one per position feed 32 multiply-adds per position
 // (48 to 64 clk of shared memory for 32 to 64 of the FP32 pipe; 4 positions x 4
-// channels, 32 clk for 16, spent 68 k of a tile-step's 70 k clk on loads by this count).  Multiply-adds run as FP32
-// pairs over channels, rounded like fmaf, in one chain over taps, then input channels.
+// channels, 32 clk for 16, spent 68 k of a tile-step's 70 k clk on loads by this
+// count).  Multiply-adds run as FP32 pairs over channels, rounded like fmaf, in one
+// chain over taps, then input channels.
 // Activations lie by groups of four channels, [group][position]: consecutive positions
 // are consecutive 16-byte words.  A layer's outputs stay in registers until every warp
 // has read its inputs and then replace them, so that one activation buffer serves all
