@@ -112,7 +112,7 @@ evsnet_pix16_kernel(Pix16Params P, const float* __restrict__ logl, const float* 
       if (ks0 == 0 && s < S) xnext = frame(P.f0 + s, ql) - frame(P.f0 + s - 1, ql);   // Eq. 1
     };
     load_x(0);
-    asm volatile("cp.async.wait_all;" ::: "memory");   // the first barrier below shows every thread's copies
+    asm volatile("cp.async.wait_all;" ::: "memory");   // the first step's barrier shows every thread's copies
     int base = hk < R ? hk : 0;    // ring position of the chunk's first step (step s at (s + hk) mod R)
     for (int s0 = 0; s0 < S; s0 += kT) {
       const int tc = min(kT, S - s0);
@@ -326,6 +326,10 @@ int et_evsnet_forward_pix16(const float* logl, int32_t F, const et_evsnet_weight
   P.R = P.kt - 1 + kT;
   P.beta = net->beta; P.vth = net->vth; P.reset = net->reset;
   P.H = st->H; P.W = st->W; P.F = F; P.f0 = st->initialized ? 0 : 1; P.t0 = t0;
+  // a fresh state's first frame alone is no step: membrane and history stay as
+  // they are.  The kernel counts on a step: its copies of the history become
+  // visible to the warps that write it back at a step's barrier.
+  if (P.F <= P.f0) return ET_OK;
   int wo = 0;
   const int taps0 = P.ks0 > 0 ? P.ks0 * P.ks0 : P.kt;
   for (int l = 0; l < P.L; ++l) {
