@@ -403,8 +403,9 @@ int et_train_workspace_bytes(const et_evsnet_weights* net, const et_train_shape*
  * [B][ceil(K / ckpt_every)][H][W], optional I_out float [B][K][H][W].
  * Errors: ET_ERR_ARG, ET_ERR_UNIMPLEMENTED (a form other than the two above,
  * C > 16, dtype other than ET_F32 / ET_BF16 or ET_BF16 for the temporal form,
- * ckpt_every > 32), ET_ERR_CUDA.  With ET_BF16, a tensor-core wait that runs
- * out of its bound (et_set_wait_budget) leaves NaN in the affected outputs. */
+ * ckpt_every > 32), ET_ERR_CUDA.  With ET_BF16, and with ET_F32 in the temporal
+ * form of 16 channels, a wait that runs out of its bound (et_set_wait_budget)
+ * leaves NaN in the affected outputs. */
 int et_evsnet_train_forward(const float* logl, const et_train_shape* shape,
                             const et_evsnet_weights* net, int8_t* spikes, float* S_on,
                             float* S_off, float* V_ckpt, float* I_out, void* workspace,
@@ -486,8 +487,10 @@ uint64_t et_kernel_launches(void);
  * returns; the context stays usable.  The call's previous-frame buffer and
  * `initialized` flag are still updated (the host does not see the timeout until
  * it reads the count): restore the state from a copy before retrying.
- * The BF16 training convolutions bound their waits the same way; on expiry
- * they write NaN into the outputs they own (activations, currents, gradients).
+ * The training convolutions that wait (BF16: for MMAs and tile copies; FP32
+ * temporal form of 16 channels: for tile copies) bound their waits the same way;
+ * on expiry they write NaN into the outputs they own (activations, currents,
+ * gradients).
  * et_set_wait_budget(polls) sets the first bound for launches made afterwards in
  * this process: polls >= 0 sets it (0 gives up at once and forces the timeout
  * path, for testing the detection), polls < 0 restores the default.  (A poll

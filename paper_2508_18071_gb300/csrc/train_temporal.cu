@@ -833,7 +833,7 @@ tconv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, i
 // warp), 720 instructions per 1024 cycles of the FP32 pipe.
 constexpr int kStepChunk = 8;
 constexpr int kRing = 3 * kStepChunk;
-constexpr uint32_t kTmaPolls = 1u << 24;   // bound of the waits for a box
+constexpr uint32_t kDrainIters = 1u << 22;   // bound of the waits for boxes in flight after a wait gave up
 
 struct F32ConvArgs {
   int K, kt;
@@ -848,6 +848,7 @@ struct F32ConvArgs {
   const float* wp;
   const float* bp;
   float* I;
+  uint32_t wait_iters;
 };
 
 template <bool kBwd>
@@ -869,10 +870,13 @@ tconv16_tma(const __grid_constant__ CUtensorMap m_in, F32ConvArgs A) {
   // processing order u = 0 .. K-1 is time s = u (forward) or s = K-1-u (data gradient)
   auto step_of = [&](int u) { return kBwd ? K - 1 - u : u; };
   // chunk t lives in group (t - t0 + 1) mod 3; thread 0 requests its boxes
+  uint32_t asked = 0, asked_odd = 0;     // thread 0: groups requested, and those requested an odd number of times
   auto load_chunk = [&](int64_t t) {
     const int64_t sg = t / nch;
     const int c = (int)(t - sg * nch), tile = (int)(sg % A.tiles), bc = (int)(sg / A.tiles);
     const int g = (int)((t - t0 + 1) % 3), n = min(kStepChunk, K - kStepChunk * c);
+    asked |= 1u << g;
+    asked_odd ^= 1u << g;
     mbar_arrive_expect_tx(&bar[g], (uint32_t)(n * kBox));
     for (int j = 0; j < n; ++j)
       tma_load_3d(sm + (g * kStepChunk + j) * kBox, &m_in, 0, tile * kBoxPix, bc * K + step_of(kStepChunk * c + j),
@@ -885,19 +889,20 @@ tconv16_tma(const __grid_constant__ CUtensorMap m_in, F32ConvArgs A) {
     if (t0 + 1 < t1) load_chunk(t0 + 1);
   }
   uint32_t phase = 0;
-  bool ok = true;
-  if (mid) { ok = mbar_wait(&bar[0], 0, kTmaPolls); phase ^= 1u; }
+  bool ok = true, bail = false;
+  if (mid) { ok = mbar_wait(&bar[0], 0, A.wait_iters); phase ^= 1u; }
   int64_t seg = t0 / nch;
   int c = (int)(t0 - seg * nch), tile = (int)(seg % A.tiles), bc = (int)(seg / A.tiles);
   int g = 1;
-  for (int64_t t = t0; t < t1; ++t) {
+  int64_t t = t0;
+  while (t < t1) {
     const int gp = g == 0 ? 2 : g - 1;   // the previous chunk's group
     if (c == 0) {                        // steps before the clip are zero
       uint4* z = reinterpret_cast<uint4*>(sm + (gp * kStepChunk + kStepChunk - (kt - 1)) * kBox);
       for (int i = tid; i < (kt - 1) * kBox / 16; i += 256) z[i] = make_uint4(0, 0, 0, 0);
       __syncthreads();
     }
-    ok &= mbar_wait(&bar[g], (phase >> g) & 1u, kTmaPolls);
+    ok &= mbar_wait(&bar[g], (phase >> g) & 1u, A.wait_iters);
     phase ^= 1u << g;
     const int u0 = kStepChunk * c + 4 * half;
     const int64_t p = (int64_t)tile * kBoxPix + px;
@@ -973,16 +978,16 @@ tconv16_tma(const __grid_constant__ CUtensorMap m_in, F32ConvArgs A) {
                 v[i] = fmaxf(v[i], 0.0f);
                 if (A.I) Iv = fmaf(__ldg(A.wp + 4 * j + i), v[i], Iv);
               }
-              if (!ok) v[i] = __int_as_float(0x7fc00000);   // a box never came
             }
             reinterpret_cast<float4*>(A.out + idx[s] * 16)[j] = make_float4(v[0], v[1], v[2], v[3]);
           }
-          if (!kBwd && A.I) A.I[idx[s]] = ok ? Iv : __int_as_float(0x7fc00000);
+          if (!kBwd && A.I) A.I[idx[s]] = Iv;
         }
       }
     }
     fence_proxy_async_smem();
-    __syncthreads();
+    bail = __syncthreads_or(!ok) != 0;
+    if (bail) break;
     // the previous chunk's group is free for the chunk after the next
     if (tid == 0 && t + 2 < t1) load_chunk(t + 2);
     g = g == 2 ? 0 : g + 1;
@@ -990,7 +995,26 @@ tconv16_tma(const __grid_constant__ CUtensorMap m_in, F32ConvArgs A) {
       c = 0;
       if (++tile == A.tiles) { tile = 0; ++bc; }
     }
+    ++t;
   }
+  if (!bail) return;
+  // a box did not come within the bound: this chunk and those left become NaN, so
+  // that the loss shows the failure, and the boxes in flight are waited for
+  // (bounded) before the shared memory is given back
+  const float nan = __int_as_float(0x7fc00000);
+  for (; t < t1; ++t) {
+    seg = t / nch;
+    c = (int)(t - seg * nch); tile = (int)(seg % A.tiles); bc = (int)(seg / A.tiles);
+    const int64_t p = (int64_t)tile * kBoxPix + px;
+    for (int u = kStepChunk * c + 4 * half; p < A.hw && u < min(K, kStepChunk * c + 4 * half + 4); ++u) {
+      const int64_t idx = ((int64_t)bc * K + step_of(u)) * A.hw + p;
+      for (int j = 0; j < 4; ++j) reinterpret_cast<float4*>(A.out + idx * 16)[j] = make_float4(nan, nan, nan, nan);
+      if (!kBwd && A.I) A.I[idx] = nan;
+    }
+  }
+  if (tid == 0)
+    for (int i = 0; i < 3; ++i)
+      if ((asked >> i) & 1u) mbar_wait(&bar[i], ((asked_odd >> i) & 1u) ^ 1u, kDrainIters);
 }
 
 // Weight gradient: grad w[co][ci][tau] += sum dz[k][co] in[k - kt + 1 + tau][ci],
@@ -1115,7 +1139,8 @@ int launch_conv_tma(bool data_grad, const float* in, int B, int K, int64_t hw, i
                     const float* b, const float* extra, const float* mask, float* out, const float* wp,
                     const float* bp, float* I, cudaStream_t st) {
   const int64_t tiles = (hw + kBoxPix - 1) / kBoxPix, nch = (K + kStepChunk - 1) / kStepChunk;
-  F32ConvArgs A{K, kt, hw, (int)tiles, (int)nch, B * tiles * nch, w, b, extra, mask, out, wp, bp, I};
+  F32ConvArgs A{K, kt, hw, (int)tiles, (int)nch, B * tiles * nch, w, b, extra, mask, out, wp, bp, I,
+                et_tc_wait_iters()};
   CUtensorMap m_in;
   ET_TRY(map_rows(&m_in, in, (int64_t)B * K, hw));
   int nsm = 0;
