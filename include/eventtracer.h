@@ -394,7 +394,9 @@ typedef struct { int32_t B, K, H, W, ckpt_every; } et_train_shape;
 /* Bytes of the caller-allocated device workspace the two calls below need:
  * spatial form: the activations of one segment plus its gradients (about
  * (2 n_layers + 2) C B ckpt_every H W floats); temporal form: the activations
- * of the whole clip (about (n_layers + 3) C B K H W floats). */
+ * of the whole clip (about (n_layers + 3) C B K H W floats).  The workspace
+ * starts on a 4-byte boundary (else ET_ERR_ARG); in the temporal form of 16
+ * channels one off 16-byte boundaries is slower. */
 int et_train_workspace_bytes(const et_evsnet_weights* net, const et_train_shape* shape,
                              size_t* bytes);
 

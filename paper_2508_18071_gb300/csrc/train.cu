@@ -753,6 +753,7 @@ extern "C" int et_evsnet_train_forward(const float* logl, const et_train_shape* 
   if (rc != ET_OK) return rc;
   if (!logl || !spikes || !V_ckpt || !workspace || ((S_on == nullptr) != (S_off == nullptr)))
     return ET_ERR_ARG;
+  if (reinterpret_cast<uintptr_t>(workspace) % sizeof(float) != 0) return ET_ERR_ARG;
   if (et_train_is_temporal(net)) {
     if (ws_bytes < et_train_temporal_bytes(net, sh)) return ET_ERR_ARG;
     return et_train_temporal_forward(logl, sh, net, spikes, S_on, S_off, V_ckpt, I_out, workspace,
@@ -801,6 +802,7 @@ extern "C" int et_evsnet_train_backward(const float* logl, const et_train_shape*
   int rc = check(net, sh);
   if (rc != ET_OK) return rc;
   if (!logl || !V_ckpt || !dS_on || !dS_off || !grad_w || !grad_b || !workspace) return ET_ERR_ARG;
+  if (reinterpret_cast<uintptr_t>(workspace) % sizeof(float) != 0) return ET_ERR_ARG;
   if (et_train_is_temporal(net)) {
     if (ws_bytes < et_train_temporal_bytes(net, sh)) return ET_ERR_ARG;
     return et_train_temporal_backward(logl, sh, net, V_ckpt, dS_on, dS_off, alpha, grad_w, grad_b,

@@ -37,7 +37,8 @@
 //
 // With C = 16 channels a pixel-step is one 64-byte row, and both kernels have a
 // second form (tct_conv16, tct_wgrad16) that moves whole tiles by TMA and keeps
-// its CTAs resident over many tiles; the forms above serve C < 16.
+// its CTAs resident over many tiles; the forms above serve C < 16 and tensors
+// that don't start on a 16-byte boundary, which TMA can't address.
 #include "et_internal.cuh"
 #include "evsnet_common.h"
 #include "tc_ptx.cuh"
@@ -63,23 +64,9 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 }
 
 // a pixel-step's CP channels (zero beyond C) from FP32 global memory
-template <bool kC16>
 __device__ __forceinline__ void load16(const float* __restrict__ src, int C, bool ok, float (&x)[CP]) {
-  if (!ok) {
 #pragma unroll
-    for (int c = 0; c < CP; ++c) x[c] = 0.0f;
-    return;
-  }
-  if (kC16) {
-#pragma unroll
-    for (int j = 0; j < CP / 4; ++j) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(src) + j);
-      x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < CP; ++c) x[c] = c < C ? __ldg(src + c) : 0.0f;
-  }
+  for (int c = 0; c < CP; ++c) x[c] = ok && c < C ? __ldg(src + c) : 0.0f;
 }
 
 // row m of a ring slot: channels 0-7 in plane 0, 8-15 in plane 1
@@ -110,7 +97,7 @@ struct ConvArgs {
   uint32_t wait_iters;
 };
 
-template <bool kBwd, bool kC16>
+template <bool kBwd>
 __global__ void __launch_bounds__(TP)
 tct_conv(ConvArgs A) {
   extern __shared__ __align__(1024) unsigned char sm[];
@@ -164,7 +151,7 @@ tct_conv(ConvArgs A) {
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int u = 2 * c + j;
-      load16<kC16>(A.in + (live && u < K ? row(step_of(u)) : 0) * C, C, live && u < K, nx[j]);
+      load16(A.in + (live && u < K ? row(step_of(u)) : 0) * C, C, live && u < K, nx[j]);
     }
   };
   load_chunk(0);
@@ -222,13 +209,9 @@ tct_conv(ConvArgs A) {
           v[co] = z;
         }
       }
-      if (kC16) {
 #pragma unroll
-        for (int q = 0; q < CP / 4; ++q)
-          reinterpret_cast<float4*>(o)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-      } else {
-        for (int co = 0; co < C; ++co) o[co] = v[co];
-      }
+      for (int co = 0; co < CP; ++co)
+        if (co < C) o[co] = v[co];
       if (!kBwd && A.I) A.I[row(s)] = Iv;
     }
     tc_fence_before();
@@ -262,7 +245,6 @@ __device__ __forceinline__ void st_bf16(unsigned char* p, float v) {
   *reinterpret_cast<__nv_bfloat16*>(p) = __float2bfloat16_rn(v);
 }
 
-template <bool kC16>
 __global__ void __launch_bounds__(TP)
 tct_wgrad(const float* __restrict__ dz, const float* __restrict__ in, int B, int K, int64_t hw, int C,
           int kt, float* __restrict__ gw, float* __restrict__ gb, uint32_t wait_iters) {
@@ -295,8 +277,8 @@ tct_wgrad(const float* __restrict__ dz, const float* __restrict__ in, int B, int
 #pragma unroll
   for (int c = 0; c < CP; ++c) gbp[c] = 0.0f;
   float nx[CP], nd[CP];
-  load16<kC16>(in + (live ? row(0) : 0) * C, C, live, nx);
-  load16<kC16>(dz + (live ? row(0) : 0) * C, C, live, nd);
+  load16(in + (live ? row(0) : 0) * C, C, live, nx);
+  load16(dz + (live ? row(0) : 0) * C, C, live, nd);
   uint32_t phase = 0;
   for (int k = 0; k < K; ++k) {
     // stage step k: input at slots k % 8 and k % 8 + 8, dz^T
@@ -323,8 +305,8 @@ tct_wgrad(const float* __restrict__ dz, const float* __restrict__ in, int B, int
       umma_commit(&mma_bar);
     }
     if (k + 1 < K) {
-      load16<kC16>(in + (live ? row(k + 1) : 0) * C, C, live, nx);
-      load16<kC16>(dz + (live ? row(k + 1) : 0) * C, C, live, nd);
+      load16(in + (live ? row(k + 1) : 0) * C, C, live, nx);
+      load16(dz + (live ? row(k + 1) : 0) * C, C, live, nd);
     }
     const bool ok = mbar_wait(&mma_bar, phase, wait_iters);
     phase ^= 1;
@@ -856,8 +838,7 @@ int et_train_tct_conv(const float* in, int B, int K, int64_t hw, int C, int kt, 
     ET_CHECK_LAUNCH();
     return ET_OK;
   };
-  if (data_grad) return C == CP ? launch(tct_conv<true, true>) : launch(tct_conv<true, false>);
-  return C == CP ? launch(tct_conv<false, true>) : launch(tct_conv<false, false>);
+  return data_grad ? launch(tct_conv<true>) : launch(tct_conv<false>);
 }
 
 int et_train_tct_wgrad(const float* dz, const float* in, int B, int K, int64_t hw, int C, int kt, float* gw,
@@ -881,7 +862,7 @@ int et_train_tct_wgrad(const float* dz, const float* in, int B, int K, int64_t h
   const size_t smem = (size_t)kWABytes + kWBBytes;
   const int64_t blocks = (int64_t)B * ((hw + TP - 1) / TP);
   if (blocks > 0x7FFFFFFF) return ET_ERR_ARG;
-  auto kern = C == CP ? tct_wgrad<true> : tct_wgrad<false>;
+  auto kern = tct_wgrad;
   ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<(unsigned)blocks, TP, smem, st>>>(dz, in, B, K, hw, C, kt, gw, gb, et_tc_wait_iters());
   ET_CHECK_LAUNCH();

@@ -50,8 +50,9 @@ constexpr int kMaxStem = 7;
 
 // ReLU of a warp's 32 rows (lane = pixel idx0 + lane, `n` of them in the image)
 // to out; a one-layer network also writes the projection I = bp + wp . out.
-// stage: the warp's 2 KB.
-__device__ __forceinline__ void store_rows(float (&acc)[kMaxC], int64_t idx0, int n, int C, float* stage,
+// stage: the warp's 2 KB.  vec: 16 channels and 16-byte aligned rows (here and
+// below; otherwise rows are read and written a word at a time).
+__device__ __forceinline__ void store_rows(float (&acc)[kMaxC], int64_t idx0, int n, int C, bool vec, float* stage,
                                            float* __restrict__ out, const float* __restrict__ wp,
                                            const float* __restrict__ bp, float* __restrict__ I) {
   const int lane = threadIdx.x & 31;
@@ -64,7 +65,7 @@ __device__ __forceinline__ void store_rows(float (&acc)[kMaxC], int64_t idx0, in
       if (c < C) Iv = fmaf(wp[c], acc[c], Iv);
     I[idx0 + lane] = Iv;
   }
-  if (C == kMaxC) {
+  if (vec) {
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -112,7 +113,7 @@ __device__ __forceinline__ void stage_taps(float (*sw)[kMaxC], float* sb, const 
 constexpr int kWalk = 16;
 template <int T>
 __global__ void __launch_bounds__(128)
-tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, int kt,
+tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, bool vec, int kt,
           const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
           const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
   __shared__ __align__(16) float sw[kMaxKt][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
@@ -148,7 +149,7 @@ tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, int k
 #pragma unroll
     for (int t = 0; t < T; ++t)
       if (t >= tau0) fma_tap(sw[t - (T - kt)], xs[t], acc);
-    store_rows(acc, ((int64_t)bc * K + k) * hw + p0, n, C, stage[warp], out, wp, bp, I);
+    store_rows(acc, ((int64_t)bc * K + k) * hw + p0, n, C, vec, stage[warp], out, wp, bp, I);
   }
 }
 
@@ -175,7 +176,7 @@ struct Rows3 {
 };
 
 __global__ void __launch_bounds__(128)
-tstem3_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C,
+tstem3_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C, bool vec,
            const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
            const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
   __shared__ __align__(16) float sw[9][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
@@ -208,7 +209,8 @@ tstem3_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C,
       // taps outside the image: no product
       if ((t >= 3 || up) && (t < 6 || dn) && (t % 3 != 0 || R.lft) && (t % 3 != 2 || R.rgt)) fma_tap(sw[t], v, acc);
     }
-    store_rows(acc, (int64_t)bk * hw + (int64_t)y * W + x0, min(32, W - x0), C, stage[warp], out, wp, bp, I);
+    store_rows(acc, (int64_t)bk * hw + (int64_t)y * W + x0, min(32, W - x0), C, vec, stage[warp], out,
+               wp, bp, I);
 #pragma unroll
     for (int t = 0; t < 3; ++t) { r0[t] = r1[t]; r1[t] = r2[t]; r2[t] = nx[t]; }
   }
@@ -216,7 +218,7 @@ tstem3_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C,
 
 // the other stem sizes, one thread per pixel-step
 __global__ void __launch_bounds__(128)
-tstem_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C, int ks0,
+tstem_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C, bool vec, int ks0,
           const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
           const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
   __shared__ __align__(16) float sw[kMaxStem * kMaxStem][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
@@ -243,7 +245,7 @@ tstem_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C, int
       }
     }
     __syncwarp();
-    store_rows(acc, (int64_t)bk * hw + p0, (int)min((int64_t)32, hw - p0), C, stage[warp], out, wp, bp, I);
+    store_rows(acc, (int64_t)bk * hw + p0, (int)min((int64_t)32, hw - p0), C, vec, stage[warp], out, wp, bp, I);
   }
 }
 
@@ -313,15 +315,15 @@ __global__ void tbilif_bwd(const float* __restrict__ I, int B, int K, int64_t hw
 // Bound by HBM (132 bytes per pixel-step): four lanes per pixel-step, 16-byte
 // accesses (8 clips x 64 steps x 128 x 128: 0.57 -> 0.19 ms).
 // a quad's channels 4 g .. of row idx (zero beyond C)
-__device__ __forceinline__ float4 load_quad(const float* __restrict__ src, int64_t idx, int g, int C) {
-  if (C == kMaxC) return __ldg(reinterpret_cast<const float4*>(src + idx * kMaxC) + g);
+__device__ __forceinline__ float4 load_quad(const float* __restrict__ src, int64_t idx, int g, int C, bool vec) {
+  if (vec) return __ldg(reinterpret_cast<const float4*>(src + idx * kMaxC) + g);
   const float* r = src + idx * C + 4 * g;
   return make_float4(4 * g < C ? r[0] : 0.0f, 4 * g + 1 < C ? r[1] : 0.0f, 4 * g + 2 < C ? r[2] : 0.0f,
                      4 * g + 3 < C ? r[3] : 0.0f);
 }
 
 __global__ void __launch_bounds__(256)
-tproj_bwd(const float* __restrict__ dI, const float* __restrict__ h, int64_t n, int C,
+tproj_bwd(const float* __restrict__ dI, const float* __restrict__ h, int64_t n, int C, bool vec,
           const float* __restrict__ wp, float* __restrict__ dz, float* __restrict__ gwp,
           float* __restrict__ gbp) {
   __shared__ float red[8][kMaxC + 1];
@@ -332,7 +334,7 @@ tproj_bwd(const float* __restrict__ dI, const float* __restrict__ h, int64_t n, 
 #pragma unroll 4
   for (int64_t i = (int64_t)blockIdx.x * 64 + (threadIdx.x >> 2); i < n; i += (int64_t)gridDim.x * 64) {
     const float d = dI[i];
-    const float4 a = load_quad(h, i, g, C);
+    const float4 a = load_quad(h, i, g, C, vec);
     const float av[4] = {a.x, a.y, a.z, a.w};
     float z[4];
     accd += d;
@@ -341,7 +343,7 @@ tproj_bwd(const float* __restrict__ dI, const float* __restrict__ h, int64_t n, 
       acc[j] += d * av[j];
       z[j] = av[j] > 0.0f ? d * wv[j] : 0.0f;
     }
-    if (C == kMaxC) {
+    if (vec) {
       *reinterpret_cast<float4*>(dz + i * kMaxC + 4 * g) = make_float4(z[0], z[1], z[2], z[3]);
     } else {
 #pragma unroll
@@ -404,8 +406,9 @@ struct QuadRing {
   const float* src;
   int64_t idx0, step;                      // row of step j: idx0 + j step
   int g, C, n;
+  bool vec;
   __device__ __forceinline__ void request(int j) {
-    if (C == kMaxC && j < n)
+    if (vec && j < n)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
                        (uint32_t)__cvta_generic_to_shared(slot + (j & (kAhead - 1)) * 256)),
                    "l"(src + (idx0 + j * step) * kMaxC + 4 * g)
@@ -419,7 +422,7 @@ struct QuadRing {
   // row j (in order), requesting row j + kAhead - 1
   __device__ __forceinline__ float4 take(int j) {
     request(j + kAhead - 1);
-    if (C != kMaxC) return load_quad(src, idx0 + j * step, g, C);
+    if (!vec) return load_quad(src, idx0 + j * step, g, C, false);
     asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
     return slot[(j & (kAhead - 1)) * 256];
   }
@@ -435,7 +438,7 @@ constexpr int kWalkB = 32;
 template <int T>
 __global__ void __launch_bounds__(256, 2)
 tconv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K,
-                 int64_t hw, int C, int kt, float* __restrict__ gw, float* __restrict__ gb) {
+                 int64_t hw, int C, bool vec, int kt, float* __restrict__ gw, float* __restrict__ gb) {
   __shared__ float4 ring[kAhead * 256];
   const int g = threadIdx.x & 3, pl = (threadIdx.x & 31) >> 2;
   float acc[T][4] = {}, bias[4] = {};
@@ -447,7 +450,7 @@ tconv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, i
     const int k0 = (int)(it / groups % segs) * kWalkB, bc = (int)(it / groups / segs);
     if (p >= hw) continue;
     const int n = min(kWalkB, K - k0);
-    QuadRing rows{ring + threadIdx.x, dz, ((int64_t)bc * K + k0) * hw + p, hw, g, C, n};
+    QuadRing rows{ring + threadIdx.x, dz, ((int64_t)bc * K + k0) * hw + p, hw, g, C, n, vec};
     rows.start();
     const float* lf = logl + (int64_t)bc * (K + 1) * hw + p;
     float xs[T];                          // X of steps k - T + 1 .. k
@@ -491,7 +494,7 @@ tconv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, i
 constexpr int kRowsB = 32;
 __global__ void __launch_bounds__(256, 2)
 tstem3_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K, int H,
-                  int W, int C, float* __restrict__ gw, float* __restrict__ gb) {
+                  int W, int C, bool vec, float* __restrict__ gw, float* __restrict__ gb) {
   __shared__ float4 ring[kAhead * 256];
   const int g = threadIdx.x & 3, pl = (threadIdx.x & 31) >> 2;
   float acc[9][4] = {}, bias[4] = {};
@@ -505,7 +508,7 @@ tstem3_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, 
     const float* l1 = logl + ((int64_t)(bk / K) * (K + 1) + bk % K + 1) * hw + x;
     const Rows3 R{l1, l1 - hw, H, W, x > 0, x + 1 < W};
     const int n = min(kRowsB, H - y0);
-    QuadRing rows{ring + threadIdx.x, dz, bk * hw + (int64_t)y0 * W + x, W, g, C, n};
+    QuadRing rows{ring + threadIdx.x, dz, bk * hw + (int64_t)y0 * W + x, W, g, C, n, vec};
     rows.start();
     float r0[3], r1[3], r2[3], r3[3];
     R.load(y0 - 1, r0);
@@ -601,9 +604,10 @@ tstem_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, i
 }
 
 // ------------------------------------------- C -> C layers, vectorised weights
-// The layers with C < 16 input channels: weights staged as [tau][input][output],
+// The layers with C < 16 input channels, or whose rows lie off 16-byte
+// boundaries: weights staged as [tau][input][output],
 // zero-padded to 16 x 16 per tap, so that one 16-byte shared load (the same
-// address for the whole warp) feeds four FMAs.  (C = 16: the kernels below.)
+// address for the whole warp) feeds four FMAs.  (C = 16 otherwise: the kernels below.)
 constexpr int CP = 16;
 
 __device__ __forceinline__ void load_ch(const float* __restrict__ src, int C, float (&x)[CP]) {
@@ -1177,6 +1181,7 @@ struct TWorkspace {
   float* dI;
   float* g[3];              // [B][K][hw][C] gradient buffers
   size_t bytes;
+  bool vec;                 // 16 channels and rows on 16-byte boundaries
 };
 
 void tlayout(const et_evsnet_weights* net, const et_train_shape* sh, char* base, TWorkspace* ws) {
@@ -1192,6 +1197,7 @@ void tlayout(const et_evsnet_weights* net, const et_train_shape* sh, char* base,
   ws->dI = take(sizeof(float) * n);
   for (int j = 0; j < 3; ++j) ws->g[j] = take(sizeof(float) * n * net->C);
   ws->bytes = off;
+  ws->vec = net->C == kMaxC && (reinterpret_cast<uintptr_t>(base) & 15) == 0;
 }
 
 // all layers over the whole clip: activations and I
@@ -1206,16 +1212,16 @@ int tforward(const float* logl, const et_train_shape* sh, const et_evsnet_weight
   float* I0 = L == 1 ? ws.I : nullptr;
   if (net->ks0 == 3) {
     const int64_t items = (int64_t)sh->B * sh->K * ((sh->H + kRows - 1) / kRows) * ((sh->W + 31) / 32);
-    tstem3_fwd<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, net->w, net->b,
-                                                           ws.act[0], wp, bp, I0);
+    tstem3_fwd<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, ws.vec, net->w,
+                                                           net->b, ws.act[0], wp, bp, I0);
   } else if (net->ks0 > 0) {
     const dim3 grid((unsigned)((hw + 127) / 128), (unsigned)std::min<int64_t>((int64_t)sh->B * sh->K, 65535));
-    tstem_fwd<<<grid, 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, net->ks0, net->w, net->b, ws.act[0], wp,
-                                    bp, I0);
+    tstem_fwd<<<grid, 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, ws.vec, net->ks0, net->w, net->b,
+                                    ws.act[0], wp, bp, I0);
   } else {
     const int64_t items = (int64_t)sh->B * ((sh->K + kWalk - 1) / kWalk) * ((hw + 31) / 32);
     (kt <= 7 ? tconv_fwd<7> : tconv_fwd<9>)<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(
-        logl, sh->B, sh->K, hw, C, kt, net->w, net->b, ws.act[0], wp, bp, I0);
+        logl, sh->B, sh->K, hw, C, ws.vec, kt, net->w, net->b, ws.act[0], wp, bp, I0);
   }
   ET_CHECK_LAUNCH();
   for (int l = 1; l < L; ++l) {
@@ -1295,7 +1301,7 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
   const unsigned wgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nsm * 8, (n + kPts - 1) / kPts));
   float* dz = ws.g[0];
   const int n0 = layer0_taps(net);
-  tproj_bwd<<<nsm * 8, 256, 0, st>>>(ws.dI, ws.act[L - 1], n, C, net->w + twofs(L, C, kt, n0), dz,
+  tproj_bwd<<<nsm * 8, 256, 0, st>>>(ws.dI, ws.act[L - 1], n, C, ws.vec, net->w + twofs(L, C, kt, n0), dz,
                                      grad_w + twofs(L, C, kt, n0), grad_b + (int64_t)L * C);
   ET_CHECK_LAUNCH();
   const int wthr = twgrad_threads(kt);
@@ -1306,12 +1312,12 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
       1, std::min<int64_t>((int64_t)nsm * std::max(wblocks, 1), (n + kPts16 - 1) / kPts16));
   auto wgrad = [&](const float* d, int l) -> int {
     if (l == 0 && net->ks0 == 3)
-      tstem3_bwd_weight<<<nsm * 4, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, grad_w, grad_b);
+      tstem3_bwd_weight<<<nsm * 4, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, ws.vec, grad_w, grad_b);
     else if (l == 0 && net->ks0 > 0)
       tstem_bwd_weight<<<wgrid, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, net->ks0, grad_w, grad_b);
     else if (l == 0)
       (kt <= 7 ? tconv_bwd_weight<7> : tconv_bwd_weight<9>)<<<nsm * 4, 256, 0, st>>>(
-          d, logl, B, K, hw, C, kt, grad_w, grad_b);
+          d, logl, B, K, hw, C, ws.vec, kt, grad_w, grad_b);
     else if (net->dtype == ET_BF16)
       return et_train_tct_wgrad(d, ws.act[l - 1], B, K, hw, C, kt, grad_w + twofs(l, C, kt, n0),
                                 grad_b + (int64_t)l * C, st);
