@@ -230,8 +230,8 @@ int et_evsnet_forward_f32(const float* logl, int32_t F, const et_evsnet_weights*
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   size_t smem = 0;
   if (!plan(P, smem, max_smem)) return ET_ERR_UNIMPLEMENTED;
-  ET_CHECK_CUDA(cudaFuncSetAttribute(evsnet_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+  const int rc = et_allow_shared(evsnet_f32_kernel);
+  if (rc != ET_OK) return rc;
   dim3 grid((P.W + P.TX - 1) / P.TX, (P.H + P.TY - 1) / P.TY);
   evsnet_f32_kernel<<<grid, P.TX * P.TY, smem, stream>>>(
       P, logl, net->w, net->b, st->V, st->hist, st->last_l, events, cap,

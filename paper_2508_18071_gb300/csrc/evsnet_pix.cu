@@ -226,8 +226,8 @@ int launch(const float* logl, int32_t F, const et_evsnet_weights* net, et_evsnet
   ET_CHECK_CUDA(cudaGetDevice(&dev));
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   if ((int)smem > max_smem) return ET_ERR_UNIMPLEMENTED;
-  ET_CHECK_CUDA(cudaFuncSetAttribute(evsnet_pix_kernel<CP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+  const int rc = et_allow_shared(evsnet_pix_kernel<CP>);
+  if (rc != ET_OK) return rc;
   const int64_t npix = (int64_t)P.H * P.W;
   evsnet_pix_kernel<CP><<<(unsigned)((npix + kThreads - 1) / kThreads), kThreads, smem, stream>>>(
       P, logl, net->w, net->b, st->V, st->hist, st->last_l, events, cap,

@@ -443,7 +443,8 @@ int launch(const float* logl, int32_t F, const et_evsnet_weights* net, et_evsnet
   ET_CHECK_CUDA(cudaGetDevice(&dev));
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   if (smem + 1024 + 64 > max_smem) return ET_ERR_UNIMPLEMENTED;
-  ET_CHECK_CUDA(cudaFuncSetAttribute(evsnet_tc_kernel<CP, kF8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const int rc = et_allow_shared(evsnet_tc_kernel<CP, kF8>);
+  if (rc != ET_OK) return rc;
   const int tiles = ((P.W + TW - 1) / TW) * ((P.H + TH - 1) / TH);
   evsnet_tc_kernel<CP, kF8><<<tiles, kThreads, smem, stream>>>(
       P, logl, net->w, net->b, st->V, st->last_l, events, cap,

@@ -833,7 +833,8 @@ int et_train_tct_conv(const float* in, int B, int K, int64_t hw, int C, int kt, 
   const int64_t blocks = (int64_t)B * ((hw + TP - 1) / TP);
   if (blocks > 0x7FFFFFFF) return ET_ERR_ARG;
   auto launch = [&](auto kern) -> int {
-    ET_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int rc = et_allow_shared(kern);
+    if (rc != ET_OK) return rc;
     kern<<<(unsigned)blocks, TP, smem, st>>>(A);
     ET_CHECK_LAUNCH();
     return ET_OK;
