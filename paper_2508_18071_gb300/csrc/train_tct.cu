@@ -604,9 +604,16 @@ tct_conv16(const __grid_constant__ CUtensorMap m_in, const __grid_constant__ CUt
 // 32 TMEM columns, each always for one of them, leave the tap of every entry
 // fixed while the ring turns.  The chunks are split evenly over the resident
 // CTAs (2 per SM) as in tct_conv16; an accumulator sums a quarter of its CTA's
-// chunks, one atomic per entry and CTA follows.  Bound by HBM: 128 bytes per
-// pixel-step (8 clips x 64 x 128 x 128: 0.50 ms transposed, 0.27 with one step
-// and N = 16 per 8 MMAs on a doubled ring, now 0.182; floor 0.158).
+// chunks, one atomic per entry and CTA follows.  The MMAs' additions round
+// towards zero, so an accumulator's error grows with the length of its sum (about
+// 2^-26 per addition: at 32 clips of 64 x 256 x 256 on the resident CTAs alone 6.7e-5 of
+// the gradient's norm, tct_wgrad 7.8e-6): a CTA takes at most 2 K chunks, half of
+// tct_wgrad's sum of K steps, and larger calls whole waves of CTAs (2.64 -> 2.81 ms,
+// 6.7e-5 -> 3.2e-6).  24 chunks where K is small: the atomics' rounding, one per CTA
+// and entry, is as large there.
+// Bound by HBM: 128 bytes per pixel-step (8 clips x 64 x 128 x 128: 0.50 ms
+// transposed, 0.27 with one step and N = 16 per 8 MMAs on a doubled ring, now
+// 0.182; floor 0.158).
 constexpr int kWStage = 2;               // chunks in flight
 constexpr int kWAcc = 4;
 
@@ -851,12 +858,14 @@ int et_train_tct_wgrad(const float* dz, const float* in, int B, int K, int64_t h
     CUtensorMap m_dz, m_in;
     int rc = map_rows(&m_dz, dz, (int64_t)B * K, hw);
     if (rc == ET_OK) rc = map_rows(&m_in, in, (int64_t)B * K, hw);
-    int grid = 0;
-    if (rc == ET_OK) rc = resident_ctas(A.total, &grid);
+    int ctas = 0;
+    if (rc == ET_OK) rc = resident_ctas(A.total, &ctas);
     if (rc != ET_OK) return rc;
+    const int64_t wave = (int64_t)ctas * std::max(2 * K, 24), grid = (A.total + wave - 1) / wave * ctas;
+    if (grid > 0x7FFFFFFF) return ET_ERR_ARG;
     const size_t smem = (size_t)kWStage * 4 * kBox + 10 * kSlot;
     ET_CHECK_CUDA(cudaFuncSetAttribute(tct_wgrad16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    tct_wgrad16<<<grid, TP, smem, st>>>(m_dz, m_in, A);
+    tct_wgrad16<<<(unsigned)grid, TP, smem, st>>>(m_dz, m_in, A);
     ET_CHECK_LAUNCH();
     return ET_OK;
   }
