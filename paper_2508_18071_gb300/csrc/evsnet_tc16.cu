@@ -80,14 +80,6 @@ __device__ __forceinline__ uint32_t relu2(uint32_t v) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// 32 lanes x 16 TMEM columns of zeros
-__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
-      "r"(0u)
-      : "memory");
-}
-
 template <int S>                       // M blocks of a tile: 4, 6 or 8
 __global__ void __launch_bounds__(kThreads, 3)
 evsnet_tc16_kernel(Tc16Params P, const float* __restrict__ logl, const float* __restrict__ wg,

@@ -175,6 +175,14 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float* v) {
       : "memory");
 }
 
+// 32 lanes x 16 TMEM columns of zeros
+__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
+      "r"(0u)
+      : "memory");
+}
+
 // 32 lanes x one 32-bit TMEM column: store (complete after tmem_wait_st), and
 // three single-column loads completed by one wait inside the same statement
 __device__ __forceinline__ void tmem_st1(uint32_t taddr, float v) {

@@ -654,7 +654,11 @@ tct_wgrad16(const __grid_constant__ CUtensorMap m_dz, const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-  const uint32_t idesc = umma_idesc_bf16_mn(TP, 2 * CP);
+  // a clip's odd last step meets the ring alone (N = 16): products with the step
+  // after it would be 0 times the ring, NaN where that holds infinities
+  constexpr uint32_t idesc2 = umma_idesc_bf16_mn(TP, 2 * CP), idesc1 = umma_idesc_bf16_mn(TP, CP);
+  for (int i = 0; i < kWAcc * 2; ++i) tmem_zero16(tmem + lane_base + (uint32_t)(i * CP));
+  tmem_wait_st();
   // MN-major, no swizzle: leading offset = next 8 pixels (K), stride offset =
   // next 8 channels (the planes of consecutive slots are 2 KB apart)
   const uint64_t a_desc = umma_desc(smem_u32(ring), 128, kPlane), b_desc = umma_desc(smem_u32(dslot), 128, kPlane);
@@ -698,14 +702,10 @@ tct_wgrad16(const __grid_constant__ CUtensorMap m_dz, const __grid_constant__ CU
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
+      if (j >= n) break;
       float x[CP], d[CP];
-      if (j < n) {
-        box_load(stage + (si * 4 + j) * kBox, tid, x);
-        box_load(stage + (si * 4 + 2 + j) * kBox, tid, d);
-      } else {                           // no second step: zeros on both sides of its products
-#pragma unroll
-        for (int i = 0; i < CP; ++i) x[i] = d[i] = 0.0f;
-      }
+      box_load(stage + (si * 4 + j) * kBox, tid, x);
+      box_load(stage + (si * 4 + 2 + j) * kBox, tid, d);
       store_slot(ring + ((k + j) & 7) * kSlot, tid, x);
       store_slot(dslot + j * kSlot, tid, d);
       if (t >= t0)
@@ -722,8 +722,8 @@ tct_wgrad16(const __grid_constant__ CUtensorMap m_dz, const __grid_constant__ CU
       const int q = c & (kWAcc - 1);
       if (tid == 0) {
         for (int j = 0; j < TP / 16; ++j)
-          umma_bf16(tmem + (uint32_t)(q * 2 * CP), a_desc + (uint64_t)(j * 16), b_desc + (uint64_t)(j * 16), idesc,
-                    (((used >> q) & 1u) || j > 0) ? 1u : 0u);
+          umma_bf16(tmem + (uint32_t)(q * 2 * CP), a_desc + (uint64_t)(j * 16), b_desc + (uint64_t)(j * 16),
+                    n == 2 ? idesc2 : idesc1, 1u);
         umma_commit(&mma_bar);
       }
       used |= 1u << q;
