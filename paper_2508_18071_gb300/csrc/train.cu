@@ -513,8 +513,12 @@ conv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, in
       ulonglong2 win[3];
       win[0] = *reinterpret_cast<const ulonglong2*>(xr + slot(0, iq));
       win[1] = *reinterpret_cast<const ulonglong2*>(xr + slot(1, iq));
+      // no position right of the image: its zero times an infinity in the image's
+      // last column would be NaN
+      const int np = W - x0;
 #pragma unroll
       for (int p = 0; p < CW; ++p) {
+        if (p >= np) break;
         win[(p + 2) % 3] = *reinterpret_cast<const ulonglong2*>(xr + slot(p + 2, iq));
         const float4 d = *reinterpret_cast<const float4*>(dr + slot(p, cq));
         const f32x2 d2[4] = {pack2f(d.x, d.x), pack2f(d.y, d.y), pack2f(d.z, d.z), pack2f(d.w, d.w)};

@@ -47,3 +47,13 @@ def test_temporal(dtype, kt, K, step):
     want = np.zeros_like(got)
     want[:, CH, [t for t in range(kt) if step + kt - 1 - t < K]] = True
     np.testing.assert_array_equal(got, want)
+
+
+@pytest.mark.parametrize("H,W,y,x", [(20, 48, 5, 47), (20, 48, 0, 0), (17, 50, 16, 49), (9, 64, 8, 31), (8, 33, 7, 32)])
+def test_3x3(H, W, y, x):
+    assert torch.cuda.is_available()
+    got = _nonfinite(_lib.ET_F32, 1, 3, 2, 6, H, W, (2, y, x))
+    want = np.zeros_like(got)
+    # tap t multiplies the output at the mirrored offset
+    want[:, CH, [t for t in range(9) if 0 <= y + 1 - t // 3 < H and 0 <= x + 1 - t % 3 < W]] = True
+    np.testing.assert_array_equal(got, want)
