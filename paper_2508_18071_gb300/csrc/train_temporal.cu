@@ -107,24 +107,35 @@ __device__ __forceinline__ void stage_taps(float (*sw)[kMaxC], float* sb, const 
   __syncthreads();
 }
 
-// Temporal layer 0, taps over the last kt steps: a thread walks kWalk steps of
-// its pixel with the last T = 7 or 9 X in registers (T >= kt), one new log
+// The layer-0 kernels walk along steps or rows with their neighbours in registers:
+// long walks where there are 16 per SM, shorter ones in small calls, whose time is
+// one walk's chain of loads (the longest throughout against these, 3 x 3 stem, 1 clip
+// of 9 x 20 x 24: forward 29 -> 5.5 us, weight gradient 23 -> 9; a thread per
+// pixel-step 6.2 and 10).
+inline int walk_length(int longest, int shortest, int64_t want, int64_t others, int n) {
+  int len = longest;
+  while (len > shortest && others * ((n + len - 1) / len) < want) len /= 2;
+  return len;
+}
+
+// Temporal layer 0, taps over the last kt steps: a thread walks up to kWalk steps
+// of its pixel with the last T = 7 or 9 X in registers (T >= kt), one new log
 // value per step (4 clips x 64 x 128 x 128: 0.30 -> 0.062 ms; HBM floor 0.042).
-constexpr int kWalk = 16;
+constexpr int kWalk = 16, kWalkMin = 4;
 template <int T>
 __global__ void __launch_bounds__(128)
-tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, bool vec, int kt,
+tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, bool vec, int kt, int walk,
           const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
           const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
   __shared__ __align__(16) float sw[kMaxKt][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
   stage_taps(sw, sb, w, b, kt, C);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t groups = (uint32_t)((hw + 31) / 32), segs = (uint32_t)(K + kWalk - 1) / kWalk;
+  const uint32_t groups = (uint32_t)((hw + 31) / 32), segs = (uint32_t)(K + walk - 1) / walk;
   const uint32_t it = blockIdx.x * 4 + warp;
   if (it >= (uint32_t)B * segs * groups) return;
   const int64_t p0 = (int64_t)(it % groups) * 32, p = min(p0 + lane, hw - 1);
   const int n = (int)min((int64_t)32, hw - p0);
-  const int k0 = (int)(it / groups % segs) * kWalk, bc = (int)(it / groups / segs);
+  const int k0 = (int)(it / groups % segs) * walk, bc = (int)(it / groups / segs);
   const float* lf = logl + (int64_t)bc * (K + 1) * hw + p;
   float xs[T];                            // X of steps k - T + 1 .. k
 #pragma unroll
@@ -133,7 +144,7 @@ tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, bool 
     xs[t] = k >= 0 ? lf[(int64_t)(k + 1) * hw] - lf[(int64_t)k * hw] : 0.0f;
   }
   float prev = lf[(int64_t)k0 * hw];
-  const int ns = min(kWalk, K - k0);
+  const int ns = min(walk, K - k0);
   float nxt = lf[(int64_t)(k0 + 1) * hw];
   for (int j = 0; j < ns; ++j) {
     const int k = k0 + j;
@@ -154,7 +165,7 @@ tconv_fwd(const float* __restrict__ logl, int B, int K, int64_t hw, int C, bool 
 }
 
 // 3 x 3 spatial stem (one step, zero outside the image, taps in row-major
-// order): a thread walks kRows rows of one column of one step with the X of
+// order): a thread walks up to kRows rows of one column of one step with the X of
 // three rows x three columns in registers (8 clips x 64 steps x 128 x 128: 0.50
 // ms with 4-byte pieces written 64 bytes apart, now 0.167; HBM floor 0.084).
 constexpr int kRows = 16;
@@ -176,24 +187,24 @@ struct Rows3 {
 };
 
 __global__ void __launch_bounds__(128)
-tstem3_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C, bool vec,
+tstem3_fwd(const float* __restrict__ logl, int B, int K, int H, int W, int C, bool vec, int rows,
            const float* __restrict__ w, const float* __restrict__ b, float* __restrict__ out,
            const float* __restrict__ wp, const float* __restrict__ bp, float* __restrict__ I) {
   __shared__ __align__(16) float sw[9][kMaxC], sb[kMaxC], stage[4][32 * kMaxC];
   stage_taps(sw, sb, w, b, 9, C);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t hw = (int64_t)H * W;
-  const uint32_t groups = (uint32_t)(W + 31) / 32, strips = (uint32_t)(H + kRows - 1) / kRows;
+  const uint32_t groups = (uint32_t)(W + 31) / 32, strips = (uint32_t)(H + rows - 1) / rows;
   const uint32_t it = blockIdx.x * 4 + warp;
   if (it >= (uint32_t)B * K * strips * groups) return;
-  const int x0 = (int)(it % groups) * 32, x = min(x0 + lane, W - 1), y0 = (int)(it / groups % strips) * kRows;
+  const int x0 = (int)(it % groups) * 32, x = min(x0 + lane, W - 1), y0 = (int)(it / groups % strips) * rows;
   const uint32_t bk = it / groups / strips;
   const float* l1 = logl + ((int64_t)(bk / K) * (K + 1) + bk % K + 1) * hw + x;
   const Rows3 R{l1, l1 - hw, H, W, x > 0, x + 1 < W};
   float r0[3], r1[3], r2[3];
   R.load(y0 - 1, r0);
   R.load(y0, r1);
-  const int ny = min(kRows, H - y0);
+  const int ny = min(rows, H - y0);
   R.load(y0 + 1, r2);
   for (int j = 0; j < ny; ++j) {
     const int y = y0 + j;
@@ -429,27 +440,27 @@ struct QuadRing {
 };
 
 // Temporal layer 0: grad w[co][tau] += sum dz[k][co] X[k - kt + 1 + tau];
-// grad b[co] += sum dz[k][co].  A thread walks kWalkB steps of one pixel with
+// grad b[co] += sum dz[k][co].  A thread walks up to kWalkB steps of one pixel with
 // the last T = 7 or 9 X in registers (T >= kt; the taps before are dropped):
 // one new log value and one 16-byte row piece per step.  68 bytes per pixel-step
 // (4 clips x 64 x 128 x 128: 0.41 ms with staged pixel-steps, 0.21 without the
-// row ring, now 0.112; HBM floor 0.042).
-constexpr int kWalkB = 32;
+// row ring, now 0.101; HBM floor 0.042).
+constexpr int kWalkB = 32, kWalkBMin = 4;
 template <int T>
 __global__ void __launch_bounds__(256, 2)
 tconv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K,
-                 int64_t hw, int C, bool vec, int kt, float* __restrict__ gw, float* __restrict__ gb) {
+                 int64_t hw, int C, bool vec, int kt, int walk, float* __restrict__ gw, float* __restrict__ gb) {
   __shared__ float4 ring[kAhead * 256];
   const int g = threadIdx.x & 3, pl = (threadIdx.x & 31) >> 2;
   float acc[T][4] = {}, bias[4] = {};
   // (a clip batch that fits the device has fewer than 2^32 rows: 32-bit item numbers)
-  const uint32_t groups = (uint32_t)((hw + 7) / 8), segs = (uint32_t)(K + kWalkB - 1) / kWalkB;
+  const uint32_t groups = (uint32_t)((hw + 7) / 8), segs = (uint32_t)(K + walk - 1) / walk;
   const uint32_t items = (uint32_t)B * segs * groups;
   for (uint32_t it = blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += gridDim.x * 8) {
     const int64_t p = (int64_t)(it % groups) * 8 + pl;
-    const int k0 = (int)(it / groups % segs) * kWalkB, bc = (int)(it / groups / segs);
+    const int k0 = (int)(it / groups % segs) * walk, bc = (int)(it / groups / segs);
     if (p >= hw) continue;
-    const int n = min(kWalkB, K - k0);
+    const int n = min(walk, K - k0);
     QuadRing rows{ring + threadIdx.x, dz, ((int64_t)bc * K + k0) * hw + p, hw, g, C, n, vec};
     rows.start();
     const float* lf = logl + (int64_t)bc * (K + 1) * hw + p;
@@ -486,28 +497,28 @@ tconv_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, i
 }
 
 // 3 x 3 stem: grad w[co][tap] += sum dz[k][co] X_nbr(tap)[k]; grad b[co] += sum
-// dz[k][co].  A thread walks kRowsB rows of one column of one step with the X of
+// dz[k][co].  A thread walks up to kRowsB rows of one column of one step with the X of
 // three rows x three columns in registers: three new X (six log values) and one
 // 16-byte row piece per pixel.  68 bytes per pixel-step (8 clips x 64 x 128 x
-// 128: 1.25 ms with staged pixel-steps, 0.40 without the row ring, now 0.257;
+// 128: 1.25 ms with staged pixel-steps, 0.40 without the row ring, now 0.255;
 // HBM floor 0.084).
 constexpr int kRowsB = 32;
 __global__ void __launch_bounds__(256, 2)
 tstem3_bwd_weight(const float* __restrict__ dz, const float* __restrict__ logl, int B, int K, int H,
-                  int W, int C, bool vec, float* __restrict__ gw, float* __restrict__ gb) {
+                  int W, int C, bool vec, int walk, float* __restrict__ gw, float* __restrict__ gb) {
   __shared__ float4 ring[kAhead * 256];
   const int g = threadIdx.x & 3, pl = (threadIdx.x & 31) >> 2;
   float acc[9][4] = {}, bias[4] = {};
   const int64_t hw = (int64_t)H * W;
-  const uint32_t groups = (uint32_t)(W + 7) / 8, strips = (uint32_t)(H + kRowsB - 1) / kRowsB;
+  const uint32_t groups = (uint32_t)(W + 7) / 8, strips = (uint32_t)(H + walk - 1) / walk;
   const uint32_t items = (uint32_t)B * K * strips * groups;
   for (uint32_t it = blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += gridDim.x * 8) {
-    const int x = (int)(it % groups) * 8 + pl, y0 = (int)(it / groups % strips) * kRowsB;
+    const int x = (int)(it % groups) * 8 + pl, y0 = (int)(it / groups % strips) * walk;
     const uint32_t bk = it / groups / strips;
     if (x >= W) continue;
     const float* l1 = logl + ((int64_t)(bk / K) * (K + 1) + bk % K + 1) * hw + x;
     const Rows3 R{l1, l1 - hw, H, W, x > 0, x + 1 < W};
-    const int n = min(kRowsB, H - y0);
+    const int n = min(walk, H - y0);
     QuadRing rows{ring + threadIdx.x, dz, bk * hw + (int64_t)y0 * W + x, W, g, C, n, vec};
     rows.start();
     float r0[3], r1[3], r2[3], r3[3];
@@ -1210,18 +1221,25 @@ int tforward(const float* logl, const et_train_shape* sh, const et_evsnet_weight
   const float* wp = net->w + twofs(L, C, kt, n0);
   const float* bp = net->b + (int64_t)L * C;
   float* I0 = L == 1 ? ws.I : nullptr;
+  int nsm = 0;
+  ET_TRY(sm_count(&nsm));
+  const int64_t warps = 16ll * nsm;
   if (net->ks0 == 3) {
-    const int64_t items = (int64_t)sh->B * sh->K * ((sh->H + kRows - 1) / kRows) * ((sh->W + 31) / 32);
-    tstem3_fwd<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, ws.vec, net->w,
+    const int64_t others = (int64_t)sh->B * sh->K * ((sh->W + 31) / 32);
+    const int rows = walk_length(kRows, 1, warps, others, sh->H);
+    const int64_t items = others * ((sh->H + rows - 1) / rows);
+    tstem3_fwd<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, ws.vec, rows, net->w,
                                                            net->b, ws.act[0], wp, bp, I0);
   } else if (net->ks0 > 0) {
     const dim3 grid((unsigned)((hw + 127) / 128), (unsigned)std::min<int64_t>((int64_t)sh->B * sh->K, 65535));
     tstem_fwd<<<grid, 128, 0, st>>>(logl, sh->B, sh->K, sh->H, sh->W, C, ws.vec, net->ks0, net->w, net->b,
                                     ws.act[0], wp, bp, I0);
   } else {
-    const int64_t items = (int64_t)sh->B * ((sh->K + kWalk - 1) / kWalk) * ((hw + 31) / 32);
+    const int64_t others = (int64_t)sh->B * ((hw + 31) / 32);
+    const int walk = walk_length(kWalk, kWalkMin, warps, others, sh->K);
+    const int64_t items = others * ((sh->K + walk - 1) / walk);
     (kt <= 7 ? tconv_fwd<7> : tconv_fwd<9>)<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(
-        logl, sh->B, sh->K, hw, C, ws.vec, kt, net->w, net->b, ws.act[0], wp, bp, I0);
+        logl, sh->B, sh->K, hw, C, ws.vec, kt, walk, net->w, net->b, ws.act[0], wp, bp, I0);
   }
   ET_CHECK_LAUNCH();
   for (int l = 1; l < L; ++l) {
@@ -1311,13 +1329,25 @@ int et_train_temporal_backward(const float* logl, const et_train_shape* sh,
   const unsigned wgrid16 = (unsigned)std::max<int64_t>(
       1, std::min<int64_t>((int64_t)nsm * std::max(wblocks, 1), (n + kPts16 - 1) / kPts16));
   auto wgrad = [&](const float* d, int l) -> int {
-    if (l == 0 && net->ks0 == 3)
-      tstem3_bwd_weight<<<nsm * 4, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, ws.vec, grad_w, grad_b);
+    // layer 0: a walk per warp, the resident two blocks of 8 warps per SM (four per
+    // SM: 2 clips of 33 x 37 x 45 26 us instead of 18, as each block ends with its
+    // share of the atomics; 8 clips of 64 x 128 x 128 0.262 ms instead of 0.255)
+    const int64_t warps = 16ll * nsm;
+    auto blocks = [&](int64_t items) { return (unsigned)std::min<int64_t>((items + 7) / 8, nsm * 2); };
+    if (l == 0 && net->ks0 == 3) {
+      const int64_t others = (int64_t)B * K * ((sh->W + 7) / 8);
+      const int walk = walk_length(kRowsB, 1, warps, others, sh->H);
+      tstem3_bwd_weight<<<blocks(others * ((sh->H + walk - 1) / walk)), 256, 0, st>>>(
+          d, logl, B, K, sh->H, sh->W, C, ws.vec, walk, grad_w, grad_b);
+    }
     else if (l == 0 && net->ks0 > 0)
       tstem_bwd_weight<<<wgrid, 256, 0, st>>>(d, logl, B, K, sh->H, sh->W, C, net->ks0, grad_w, grad_b);
-    else if (l == 0)
-      (kt <= 7 ? tconv_bwd_weight<7> : tconv_bwd_weight<9>)<<<nsm * 4, 256, 0, st>>>(
-          d, logl, B, K, hw, C, ws.vec, kt, grad_w, grad_b);
+    else if (l == 0) {
+      const int64_t others = (int64_t)B * ((hw + 7) / 8);
+      const int walk = walk_length(kWalkB, kWalkBMin, warps, others, K);
+      (kt <= 7 ? tconv_bwd_weight<7> : tconv_bwd_weight<9>)<<<blocks(others * ((K + walk - 1) / walk)), 256, 0, st>>>(
+          d, logl, B, K, hw, C, ws.vec, kt, walk, grad_w, grad_b);
+    }
     else if (net->dtype == ET_BF16)
       return et_train_tct_wgrad(d, ws.act[l - 1], B, K, hw, C, kt, grad_w + twofs(l, C, kt, n0),
                                 grad_b + (int64_t)l * C, st);
