@@ -18,8 +18,8 @@ int et_evsnet_forward_tc16(const float* logl, int32_t F, const et_evsnet_weights
 int et_evsnet_forward_pix(const float* logl, int32_t F, const et_evsnet_weights* net,
                           et_evsnet_state* st, int32_t t0, et_event* events, int64_t cap,
                           int64_t* n_events, float* I_out, int8_t* spikes, cudaStream_t stream);
-// the pixel-wise form of at most 16 channels with its history in shared memory;
-// declines (before launching anything) what does not fit
+// the pixel-wise form at kt = 7 and 13 to 16 channels with its history in shared
+// memory; declines (before launching anything) what does not fit or is slower so
 int et_evsnet_forward_pix16(const float* logl, int32_t F, const et_evsnet_weights* net,
                             et_evsnet_state* st, int32_t t0, et_event* events, int64_t cap,
                             int64_t* n_events, float* I_out, int8_t* spikes, cudaStream_t stream);

@@ -243,8 +243,12 @@ int et_evsnet_forward_pix(const float* logl, int32_t F, const et_evsnet_weights*
                           int64_t* n_events, float* I_out, int8_t* spikes, cudaStream_t stream) {
   if (net->ks != 1 || net->kt > kMaxKt || net->C > 32) return ET_ERR_UNIMPLEMENTED;
   // kt = 7 with 13 to 16 channels (the networks of the configurations): the
-  // history in shared memory, where it fits (640 x 360, 16 steps of the paper's
-  // form: 4.04 ms here, bound by the history's way from L2, 2.38 there)
+  // history in shared memory, where it fits and is faster.  Same sums in the same
+  // order, so a clip may change from one kernel to the other between calls.  Other
+  // kt are not compiled there; below 13 channels its 16-channel products lose ground
+  // (12 channels, 7 layers, 8 steps of 640 x 360: 1.42 times as fast as here; 8: 1.05,
+  // behind a 3 x 3 stem 0.93; 4: 0.80) although images of less than 5000 pixels
+  // would gain there too.
   const int rc = et_evsnet_forward_pix16(logl, F, net, st, t0, events, cap, n_events, I_out, spikes, stream);
   if (rc != ET_ERR_UNIMPLEMENTED) return rc;
   if (net->C <= 16)

@@ -314,6 +314,24 @@ evsnet_pix16_kernel(Pix16Params P, const float* __restrict__ logl, const float* 
   }
 }
 
+// Whether evsnet_pix.cu takes less time for S steps.  This kernel pays for set-up
+// and history once per tile and for up to eight steps at a time, and its stem reads
+// the frames once per warp; the other one pays per step, and fills the device from
+// 256 pixels per SM on instead of 32.  Both sides are sums fitted to 300 calls of
+// each (C = 13 and 16, 2 to 7 layers, ks0 0 to 7, 1 to 32 steps, 187 x 253 to 720 x
+// 1280; ns per 1000 pixels of full waves, within 15 and 28 %): the slower side is
+// taken in few of them, by 14 % at most.  640 x 360, C = 16, here / there: 3 layers,
+// 1 step 0.35 / 0.24 ms, 8 steps 0.65 / 0.81, behind a 5 x 5 stem 1.07 / 0.79; 7
+// layers, 1 step 0.78 / 0.87, 16 steps 2.43 / 4.08.
+bool pix_is_faster(const Pix16Params& P, int S, int64_t npix, int nsm) {
+  auto waves = [&](int per) { return (npix + (int64_t)per * nsm - 1) / ((int64_t)per * nsm) * per; };
+  const int64_t l = P.L - 1, rest = S % kT;
+  const int64_t s8 = S - rest + (rest == 0 ? 0 : rest <= 2 ? 2 : rest <= 4 ? 4 : kT);   // steps as chunks run them
+  const int64_t there = 23 * l * P.C + S * (43 + (19 * l * P.C + 1) / 2);
+  const int64_t here = 520 + 295 * l + s8 * (80 + 71 * l) + P.ks0 * P.ks0 * (17 + 7 * (int64_t)S);
+  return waves(256) * there < waves(kP) * here;
+}
+
 }  // namespace
 
 int et_evsnet_forward_pix16(const float* logl, int32_t F, const et_evsnet_weights* net,
@@ -349,6 +367,7 @@ int et_evsnet_forward_pix16(const float* logl, int32_t F, const et_evsnet_weight
   ET_CHECK_CUDA(cudaGetDevice(&dev));
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  if (pix_is_faster(P, P.F - P.f0, (int64_t)P.H * P.W, nsm)) return ET_ERR_UNIMPLEMENTED;
   auto kern = evsnet_pix16_kernel;
   if (smem + sizeof(uint32_t) * kStageCap > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
   const int rc = et_allow_shared(kern);
