@@ -240,8 +240,10 @@ __device__ __forceinline__ void load_row8(const unsigned char* slot, int m, floa
 
 // kForm, the layer 0 a kernel is compiled for (one kernel for all of them is 150 KB
 // of code, more than the instruction cache, of which a round touches pieces in all
-// three worker groups): 0 temporal, 3 the 3 x 3 stem by thread loads, 4 the 3 x 3
-// stem by TMA, -1 any (calibration, other stem sizes)
+// three worker groups): 0 temporal, 1 a stem of 1, 5 or 7 (16 channels, 7
+// layers behind 5 x 5 on 253 x 187, BF16: one step 156 -> 127 us, eight about 285 -> 225
+// against the instance for any form, tap by tap), 3 the 3 x 3 stem by thread loads, 4 the 3 x 3 stem by TMA, -1 any
+// (calibration)
 template <bool kF8, bool kCal, int kForm>
 __global__ void __launch_bounds__(kThreads, 1)
 evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const float* __restrict__ logl,
@@ -255,8 +257,9 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   __shared__ uint64_t drain_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ uint32_t staged[TP / 32][kStageCap];   // group 0's events
-  const int L = P.L, C = P.C, kt = P.kt, R = P.R, hk = kt - 1, ks0 = kForm < 0 ? P.ks0 : kForm == 4 ? 3 : kForm;
+  const int L = P.L, C = P.C, kt = P.kt, R = P.R, hk = kt - 1, ks0 = kForm < 0 || kForm == 1 ? P.ks0 : kForm == 4 ? 3 : kForm;
   constexpr bool kTma = kForm == 4;
+  const bool stem3 = kForm >= 3 || (kForm < 0 && ks0 == 3), no_stem = kForm == 0 || (kForm < 0 && ks0 == 0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int p = tid & (TP - 1);         // pixel of the tile = TMEM lane
   const int grp = tid >> 7;             // worker group (4 = the issuing warp)
@@ -291,7 +294,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   float* w0 = bp + 4;                                          // [taps][CP] layer 0
   const int taps0 = ks0 > 0 ? ks0 * ks0 : kt;
   float* xh = w0 + taps0 * CP;                                 // [R][TP] layer-0 X ring (temporal layer 0)
-  float* dq = xh + (ks0 == 0 ? R * TP : 0);                    // FP8: [L][CP] weight scale, then x input scale
+  float* dq = xh + (no_stem ? R * TP : 0);                    // FP8: [L][CP] weight scale, then x input scale
   float* isc = dq + L * CP;                                    // FP8: [kMaxLayers] 1 / input scale of layer l
   float* scl = isc + kMaxLayers;                               // FP8: [kMaxLayers] input scale of layer l
   const int npairs = (kt + 2) / 2;                             // FP8: MMAs per layer (slot pairs)
@@ -470,7 +473,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
 #pragma unroll
         for (int j = 0; j < kT; ++j) xn[j][t] = l[j + 1] - l[j];
       }
-    } else if (ks0 == 3) {
+    } else if (stem3) {
 #pragma unroll
       for (int t = 0; t < 9; ++t)
 #pragma unroll
@@ -498,7 +501,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
         }
       }
     };
-    if (ks0 == 3) {
+    if (stem3) {
 #pragma unroll
       for (int t = 0; t < 9; ++t) {
         float x[kT];
@@ -506,24 +509,32 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
         for (int j = 0; j < kT; ++j) x[j] = xn[j][t];
         tap(t, x);
       }
-    } else if (ks0 > 0) {
+    } else if (!no_stem) {
       const int r0 = ks0 >> 1;
+#pragma unroll 1
       for (int dy = 0; dy < ks0; ++dy) {
         const int yy = py + dy - r0;
         if (yy < 0 || yy >= P.H) continue;
-        for (int dx = 0; dx < ks0; ++dx) {
+        // a row's frames, every load in flight at once
+        float l[kMaxStem][kT + 1];
+#pragma unroll
+        for (int dx = 0; dx < kMaxStem; ++dx) {
           const int xx = px + dx - r0;
-          if (xx < 0 || xx >= P.W) continue;
-          const int64_t qq = (int64_t)yy * P.W + xx;
+          const bool in = dx < ks0 && xx >= 0 && xx < P.W;
+          const int64_t qq = (int64_t)yy * P.W + (in ? xx : px);
+#pragma unroll
+          for (int j = 0; j <= kT; ++j) {
+            const int f = P.f0 + s0 - 1 + min(j, tc);
+            l[dx][j] = !in ? 0.0f : f < 0 ? last_l[qq] : __ldg(logl + (int64_t)f * npix + qq);
+          }
+        }
+#pragma unroll
+        for (int dx = 0; dx < kMaxStem; ++dx) {
+          const int xx = px + dx - r0;
+          if (dx >= ks0 || xx < 0 || xx >= P.W) continue;
           float x[kT];
 #pragma unroll
-          for (int j = 0; j < kT; ++j) {
-            const int f = P.f0 + s0 + j;
-            x[j] = 0.0f;
-            if (j < tc)
-              x[j] = __ldg(logl + (int64_t)f * npix + qq) -
-                     (f == 0 ? last_l[qq] : __ldg(logl + (int64_t)(f - 1) * npix + qq));
-          }
+          for (int j = 0; j < kT; ++j) x[j] = j < tc ? l[dx][j + 1] - l[dx][j] : 0.0f;
           tap(dy * ks0 + dx, x);
         }
       }
@@ -666,10 +677,10 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
       const int64_t qq = in ? (int64_t)y * P.W + x : 0;
       xbuf[i] = !in ? 0.0f : f < 0 ? last_l[qq] : __ldg(logl + (int64_t)f * npix + qq);
     }
-  } else if (ks0 == 3 && stem_part && nch > 0) {
+  } else if (stem3 && stem_part && nch > 0) {
     load_x9(0);
   }
-  if (ks0 == 0 && stem_grp)
+  if (no_stem && stem_grp)
     for (int j = 0; j < hk; ++j) xh[ring_pos(j - hk, R) * TP + p] = live ? hist[hidx(0, j, 0)] : 0.0f;
   // Rounds: in round tau tensor-core layer l computes chunk tau - l + 1 and
   // layer 0 chunk tau + 1, so that one MMA issue and one barrier serve every
@@ -743,7 +754,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
     // ---- layer 0 of the next chunk, in registers, while the MMAs run
     if (stem_part && tau + 1 < nch) {
       stem(tau + 1);
-      if (ks0 == 3 && !kTma) load_x9((tau + 2) * kT);   // consumed next round
+      if (stem3 && !kTma) load_x9((tau + 2) * kT);   // consumed next round
     }
     // ---- this group's epilogues, last layer first, each after its layer's commit
     for (int l = L - 1; l >= 1 && worker; --l) {
@@ -891,7 +902,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
       }
     }
     if (live) {
-      if (ks0 == 0 && stem_grp)
+      if (no_stem && stem_grp)
         for (int j = 0; j < hk; ++j) hist[hidx(0, j, 0)] = xh[ring_pos(S - hk + j, R) * TP + p];
     }
   }
@@ -984,14 +995,14 @@ int tct_launch(const float* logl, int32_t F, const et_evsnet_weights* net, et_ev
   int nsm = 0;
   ET_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   // static shared memory (barriers, TMEM slot, flag) comes on top of the dynamic part
-  const int form = P.tma ? 4 : (P.ks0 == 0 || P.ks0 == 3) ? P.ks0 : -1;
+  const int form = P.tma ? 4 : (P.ks0 == 0 || P.ks0 == 3) ? P.ks0 : 1;
   auto kern = evsnet_tct_kernel<false, true, -1>;
   if (!amax && f8)
     kern = form == 4 ? evsnet_tct_kernel<true, false, 4> : form == 3 ? evsnet_tct_kernel<true, false, 3>
-           : form == 0 ? evsnet_tct_kernel<true, false, 0> : evsnet_tct_kernel<true, false, -1>;
+           : form == 0 ? evsnet_tct_kernel<true, false, 0> : evsnet_tct_kernel<true, false, 1>;
   else if (!amax)
     kern = form == 4 ? evsnet_tct_kernel<false, false, 4> : form == 3 ? evsnet_tct_kernel<false, false, 3>
-           : form == 0 ? evsnet_tct_kernel<false, false, 0> : evsnet_tct_kernel<false, false, -1>;
+           : form == 0 ? evsnet_tct_kernel<false, false, 0> : evsnet_tct_kernel<false, false, 1>;
   cudaFuncAttributes fa;
   ET_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
   if (smem + fa.sharedSizeBytes > (size_t)max_smem) return ET_ERR_UNIMPLEMENTED;
