@@ -240,10 +240,9 @@ __device__ __forceinline__ void load_row8(const unsigned char* slot, int m, floa
 
 // kForm, the layer 0 a kernel is compiled for (one kernel for all of them is 150 KB
 // of code, more than the instruction cache, of which a round touches pieces in all
-// three worker groups): 0 temporal, 1 a stem of 1, 5 or 7 (16 channels, 7
-// layers behind 5 x 5 on 253 x 187, BF16: one step 156 -> 127 us, eight about 285 -> 225
-// against the instance for any form, tap by tap), 3 the 3 x 3 stem by thread loads, 4 the 3 x 3 stem by TMA, -1 any
-// (calibration)
+// three worker groups): 0 temporal, 1 a stem of 1, 5 or 7 (7 layers behind 5 x 5 on
+// 253 x 187, BF16: one step 156 us in the instance for any form, tap by tap, here 127),
+// 3 the 3 x 3 stem by thread loads, 4 the 3 x 3 stem by TMA, -1 any (calibration)
 template <bool kF8, bool kCal, int kForm>
 __global__ void __launch_bounds__(kThreads, 1)
 evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const float* __restrict__ logl,
@@ -262,7 +261,7 @@ evsnet_tct_kernel(const __grid_constant__ CUtensorMap tmap, TctParams P, const f
   const bool stem3 = kForm >= 3 || (kForm < 0 && ks0 == 3), no_stem = kForm == 0 || (kForm < 0 && ks0 == 0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int p = tid & (TP - 1);         // pixel of the tile = TMEM lane
-  const int grp = tid >> 7;             // worker group (4 = the issuing warp)
+  const int grp = tid >> 7;             // worker group (3 = the issuing warp)
   // group g runs the epilogues of the tensor-core layers l with
   // (L - 1 - l) % 3 == g (the last layer, with the projection and BiLIF, in
   // group 0), so that consecutive layers' epilogues run in different warps

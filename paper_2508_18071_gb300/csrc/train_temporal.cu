@@ -843,9 +843,11 @@ tconv16_bwd_weight(const float* __restrict__ dz, const float* __restrict__ in, i
 // and split evenly over one CTA per SM.  Steps arrive as TMA boxes (64-byte rows,
 // read by each pixel's thread without bank conflicts) in three groups of 8: the
 // previous chunk's (its last kt - 1 steps are this chunk's past), this one's and
-// the next one's.  A thread computes 4 steps of a pixel: a tap's 16 x 16 weights
-// serve 64 pair multiply-adds per 4 weight loads (the same address for the whole
-// warp), 720 instructions per 1024 cycles of the FP32 pipe.
+// the next one's.  A thread computes 4 steps of a pixel: four input channels of a tap
+// are 16 weight loads (the same address for the whole warp) and 4 input ones for 128
+// pair multiply-adds, 80 clk of shared memory (4 per 16-byte load of a warp) for 64 of
+// the FP32 pipe: shared memory bounds it (4 clips x 64 x 128 x 128: 0.35 ms forward, 0.38
+// data gradient).
 constexpr int kStepChunk = 8;
 constexpr int kRing = 3 * kStepChunk;
 constexpr uint32_t kDrainIters = 1u << 22;   // bound of the waits for boxes in flight after a wait gave up

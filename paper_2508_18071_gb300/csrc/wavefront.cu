@@ -478,7 +478,7 @@ int et_render_wavefront(et_scene* s, int n_frames, int first_frame, int W, int H
       A.box.scale[k] = ext > 0.0f ? 64.0f / ext : 0.0f;
     }
   }
-    const int grid_shade = nsm * 16;
+  const int grid_shade = nsm * 16;
   for (int f0 = 0; f0 < n_frames; f0 += frames_per_batch) {
     const int nf = std::min(frames_per_batch, n_frames - f0);
     for (int s0 = 0; s0 < spp; s0 += samples_per_batch) {
