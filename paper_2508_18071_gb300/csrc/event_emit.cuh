@@ -4,18 +4,20 @@
 
 // Every lane of the warp must call this (lanes without events pass n = 0).
 // Lane i appends n_i copies of (x, y, t, p); one atomicAdd per warp reserves
-// the slots.  Slots at or beyond `cap` are counted but not written.
+// the slots.  Slots at or beyond `cap` are counted but not written.  Sum holds the
+// warp's count: 64 bits where a lane's may be near 2^32 (an infinite step).
+template <typename Sum = uint32_t>
 __device__ __forceinline__ void emit_events_warp(et_event* events, int64_t cap,
                                                  unsigned long long* counter, uint32_t n,
                                                  uint32_t x, uint32_t y, uint32_t t, int p) {
   const unsigned lane = threadIdx.x & 31u;
-  uint32_t incl = n;
+  Sum incl = n;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    const Sum v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= (unsigned)o) incl += v;
   }
-  const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+  const Sum total = __shfl_sync(0xFFFFFFFFu, incl, 31);
   if (total == 0) return;
   unsigned long long base = 0;
   if (lane == 31) base = atomicAdd(counter, (unsigned long long)total);
@@ -95,7 +97,7 @@ struct EventStage {
       rank = (int)(incl - c);
       total = (int)__shfl_sync(0xFFFFFFFFu, incl, 31);
       if (total > kCap) {
-        emit_events_warp(events, cap, counter, cnt, x, y + dy, t0 + step, p);
+        emit_events_warp<unsigned long long>(events, cap, counter, cnt, x, y + dy, t0 + step, p);
         return;
       }
     }
